@@ -267,10 +267,13 @@ __global__ void __launch_bounds__(256, (B <= 8 ? 3 : 2)) render_bwd_kernel(const
             }
             const int count = min(B, n_items - b * B);
             if (!__all_sync(0xffffffffu, timed_out) && (uint32_t)(b * B) < wlast) {
-            for (int j = min(count, (int)(wlast - (uint32_t)(b * B))) - 1; j >= 0; --j) {
+            const int reach = min(count, (int)(wlast - (uint32_t)(b * B)));
+            for (int j0 = (B - 1) & ~31; j0 >= 0; j0 -= 32)
+            for (uint32_t hits = warp_block_hits(S.rec[buf], j0, reach, lane, bx0, by0); hits;) {
+                const int j = j0 + 31 - __clz(hits);
+                hits ^= 1u << (j - j0);
                 const uint32_t pos = (uint32_t)(b * B + j);
                 const float* rc = &S.rec[buf][j][0];
-                if (warp_block_misses(rc, bx0, by0)) continue;  // uniform per warp
                 // alpha of every lane; the warp runs the pair's gradient only if
                 // some lane contributes, and then as a whole: a lane that does not
                 // contribute carries w = 0 and dL/dalpha = 0, which makes every

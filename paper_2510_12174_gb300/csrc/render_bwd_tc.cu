@@ -457,10 +457,13 @@ __global__ void __launch_bounds__(BTC_THREADS, BTC_CTAS_PER_SM)
                 const uint32_t d1 = tmem + lane_addr + (uint32_t)((2 * bf + mt) * B);
                 const float finv = S.finv[bf];
                 if (!__all_sync(0xffffffffu, timed_out) && (uint32_t)(b * B) < wlast) {
-                    for (int j = min(count, (int)(wlast - (uint32_t)(b * B))) - 1; j >= 0; --j) {
+                    uint32_t hits = warp_block_hits(
+                        S.rec[bf], 0, min(count, (int)(wlast - (uint32_t)(b * B))), lane, bx0, by0);
+                    while (hits) {
+                        const int j = 31 - __clz(hits);
+                        hits ^= 1u << j;
                         const uint32_t pos = (uint32_t)(b * B + j);
                         const float* rc = &S.rec[bf][j][0];
-                        if (warp_block_misses(rc, bx0, by0)) continue;  // uniform per warp
                         // Gsem of this pixel and Gaussian, loaded while alpha is evaluated
                         const uint32_t gsem_raw = tmem_ld1_issue(d1 + (uint32_t)j);
                         float dx, dy, Gs, wq;

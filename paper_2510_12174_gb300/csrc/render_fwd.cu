@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(256, 2) render_fwd_kernel(const FwdParams P) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     FwdSmem<NS, B>& S = *reinterpret_cast<FwdSmem<NS, B>*>(smem_raw);
     const int tid = threadIdx.x;
-    const int warp = tid >> 5;
+    const int warp = tid >> 5, lane = tid & 31;
 
     // once per CTA: zero the semantic padding (rows shorter than NS), init barriers
     for (int j = tid; j < 2 * B * NS; j += 256) (&S.sem[0][0][0])[j] = 0.f;
@@ -179,9 +179,13 @@ __global__ void __launch_bounds__(256, 2) render_fwd_kernel(const FwdParams P) {
             const int count = min(B, n_items - b * B);
             const bool skip = __all_sync(0xffffffffu, done || timed_out);
             if (!skip) {
-                for (int j = 0; j < count; ++j) {
+#pragma unroll 1
+                for (int j0 = 0; j0 < count; j0 += 32)
+#pragma unroll 1
+                for (uint32_t hits = warp_block_hits(S.rec[buf], j0, count, lane, bx0, by0); hits;
+                     hits &= hits - 1) {
+                    const int j = j0 + __ffs(hits) - 1;
                     const float* rc = &S.rec[buf][j][0];
-                    if (warp_block_misses(rc, bx0, by0)) continue;  // uniform per warp
                     if (done) continue;
                     float dx, dy, Gs;
                     float wq;

@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(256, (B <= 16 ? 4 : 2)) render_fwd_tc_kernel(c
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Sm& S = *reinterpret_cast<Sm*>(smem_raw);
     const int tid = threadIdx.x;
-    const int warp = tid >> 5;
+    const int warp = tid >> 5, lane = tid & 31;
     constexpr uint32_t NCOLS = tmem_cols<NS>();
     constexpr uint32_t IDESC = idesc_bf16_f32(128, NS);
 
@@ -256,9 +256,12 @@ __global__ void __launch_bounds__(256, (B <= 16 ? 4 : 2)) render_fwd_tc_kernel(c
             }
             if (!skip) {
 #pragma unroll 1
-                for (int j = 0; j < count; ++j) {
+                for (int j0 = 0; j0 < count; j0 += 32)
+#pragma unroll 1
+                for (uint32_t hits = warp_block_hits(S.rec[buf], j0, count, lane, bx0, by0); hits;
+                     hits &= hits - 1) {
+                    const int j = j0 + __ffs(hits) - 1;
                     const float* rc = &S.rec[buf][j][0];
-                    if (warp_block_misses(rc, bx0, by0)) continue;  // uniform per warp
                     if (done) continue;
                     float dx, dy, Gs;
                     float wq;
