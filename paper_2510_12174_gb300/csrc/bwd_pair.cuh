@@ -52,7 +52,7 @@ __device__ __forceinline__ float bwd_pair(const float* __restrict__ rc, const Pi
     // gradient of a 200k-Gaussian test scene drifted 2.5x further
     // from the float64 reference); dL/dalpha takes an approximate
     // reciprocal
-    const float rom = __fdividef(1.f, om);
+    const float rom = rcp_ftz(om);
     if (contrib) T = __fdiv_rn(T, om);
     const float w = contrib ? alpha * T : 0.f;
     PairGeom G;
@@ -94,7 +94,7 @@ __device__ __forceinline__ float bwd_pair(const float* __restrict__ rc, const Pi
     gv[G_RGB + 2] = w * up.rgb[2];
     gv[G_K] = w * up.K;
     const float* Nw = rc + R_NW;
-    const float inv_a = __fdividef(1.f, G.a);
+    const float inv_a = rcp_ftz(G.a);
     // The Gaussian enters through v_s and d_s.  Besides g_vs the
     // record takes B = g_vs (x) w + G2 (x) d_s with w = v_s + t d_s
     // (the closest-approach point p_mid, formed without
@@ -138,7 +138,7 @@ __device__ __forceinline__ float bwd_pair(const float* __restrict__ rc, const Pi
 #pragma unroll
         for (int i = 0; i < 3; ++i) g2[i] -= G.sr * G.h * g_p[i];
         // dh/ddisc = 1 / (2 a sqrt(disc))
-        g_disc = 0.5f * g_h * inv_a * rsqrtf(G.disc);
+        g_disc = 0.5f * g_h * inv_a * rsqrt_ftz(G.disc);
         g_a -= g_h * G.h * inv_a;
     }
     // disc = a - |cv|^2
