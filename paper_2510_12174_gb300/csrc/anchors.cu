@@ -2,18 +2,24 @@
 // anchor into its M Gaussians, forward and backward.  The definitions are in
 // include/unigs_anchors.h.
 //
-// The five two-layer MLPs (F = H = 32) are tiny next to the rasterizer: about
-// 11 k multiply-adds per anchor, so one thread per anchor with every weight in
-// shared memory (broadcast reads) is the design, not the tensor cores.
+// The five two-layer MLPs (F = H = 32) are about 11 k multiply-adds per anchor
+// forward and 32 k backward, in float32; at 100k anchors of 10 Gaussians with
+// 64 logits that is 30 and 90 us of the FP32 pipes, next to 35 and 70 us for
+// the bytes.  Each layer is a product of a weight matrix with a tile of TA
+// anchors: a block of 256 threads keeps the weights, the anchors' features and
+// one branch's hidden layer in shared memory (entries [unit][anchor]), and a
+// thread owns a register tile of 4 units x TA / 32 anchors, so that 8 16-byte
+// shared loads feed 64 multiply-adds.  Outputs go through shared memory, so
+// that a warp writes whole rows: with one thread per anchor (53 KB of weights
+// read by broadcast, one multiply-add per shared load) every store of a warp
+// fell into 32 different rows, and decode and backward took 913 and 1780 us
+// at that size.  Each output still sums its terms in the same order.
 //
-// Backward: each thread recomputes its anchor's hidden layers and forms the
-// gradients of the MLP outputs from the decoded Gaussians' gradients; the
-// per-anchor gradients (position, scale, offsets, feature, base logits, base
-// k) are written by that thread.  The parameter gradients dL/dW2 = sum_a gy_a
-// (x) h_a, dL/dW1 = sum_a gpre_a (x) f_a are products over the block's 128
-// anchors, formed from shared-memory tiles by a fixed thread per entry and
-// accumulated in shared memory across the block's grid-stride iterations;
-// one float32 atomic per parameter and block adds them at the end.
+// Backward: the same tiles give the outputs, dL/dh = W2^T g_y and dL/df = W1^T
+// g_pre; the parameter gradients dL/dW2 = sum_a g_y (x) h and dL/dW1 = sum_a
+// g_pre (x) f are 4 x 4 register tiles over the block's anchors, added to
+// accumulators in shared memory tile by tile; one float32 atomic per parameter
+// and block adds them at the end.
 #include <cuda_bf16.h>
 
 #include "launch.h"
@@ -25,15 +31,21 @@ namespace {
 
 constexpr int AF = UNIGS_ANCHOR_FEAT;
 constexpr int AH = UNIGS_ANCHOR_HIDDEN;
-constexpr int ATHREADS = 128;
+constexpr int ATHREADS = 256;
 constexpr int NMLP = 5;  // sem, k, opacity, color, cov
-constexpr int MAXOUT = 7 * UNIGS_ANCHOR_MAX_OFFSETS > UNIGS_MAX_SEM ? 7 * UNIGS_ANCHOR_MAX_OFFSETS
-                                                                    : UNIGS_MAX_SEM;
 constexpr float Y00 = 0.28209479177387814f;  // 1 / (2 sqrt(pi))
+// Row stride (floats) of the weight matrices in shared memory.  No padding:
+// the 8 lanes of a shared-memory phase read the same row.
+constexpr int WS = AH;
+static_assert(AH == 32 && AF == 32, "the register tiles cover 32 hidden units");
 
-// Offsets (in floats) of each MLP's parameters in the shared-memory block.
+// Each MLP's parameters in the shared-memory block (offsets in floats; rows
+// of W1 and W2 are WS apart), its output count and its stored rows of W2: a
+// multiple of 4, the surplus zero.  The covariance branch stores the scale
+// outputs (row 3 m + i) first, then from row quat_row() the quaternions'
+// (row quat_row() + 4 m + j).
 struct WLayout {
-    int w1[NMLP], b1[NMLP], w2[NMLP], b2[NMLP], out[NMLP];
+    int w1[NMLP], b1[NMLP], w2[NMLP], b2[NMLP], out[NMLP], rows[NMLP];
     int total;
 };
 
@@ -61,115 +73,295 @@ __device__ __forceinline__ void put_feat(void* base, int64_t i, float v, bool bf
         static_cast<float*>(base)[i] = v;
 }
 
+__host__ __device__ __forceinline__ int quat_row(int M) { return (3 * M + 3) & ~3; }
+
+// Row of W2 and b2 that branch X stores as row j; -1: a row of zeros.
+__device__ __forceinline__ int param_row(int X, int out, int j, int M) {
+    if (X != 4) return j < out ? j : -1;
+    if (j < 3 * M) return 7 * (j / 3) + j % 3;
+    j -= quat_row(M);
+    return j < 0 ? -1 : 7 * (j / 4) + 3 + j % 4;
+}
+
 // Copies every MLP's parameters into shared memory (the whole block).
 __device__ void load_weights(const AnchorIn& P, const WLayout& L, float* sw) {
     for (int X = 0; X < NMLP; ++X) {
-        if (L.out[X] == 0) continue;
-        for (int i = threadIdx.x; i < AH * AF; i += blockDim.x) sw[L.w1[X] + i] = P.w1[X][i];
-        for (int i = threadIdx.x; i < AH; i += blockDim.x) sw[L.b1[X] + i] = P.b1[X][i];
-        for (int i = threadIdx.x; i < L.out[X] * AH; i += blockDim.x) sw[L.w2[X] + i] = P.w2[X][i];
-        for (int i = threadIdx.x; i < L.out[X]; i += blockDim.x) sw[L.b2[X] + i] = P.b2[X][i];
+        const int out = L.out[X];
+        if (out == 0) continue;
+        for (int i = threadIdx.x; i < AH * AF; i += ATHREADS)
+            sw[L.w1[X] + i / AF * WS + i % AF] = P.w1[X][i];
+        for (int i = threadIdx.x; i < AH; i += ATHREADS) sw[L.b1[X] + i] = P.b1[X][i];
+        for (int i = threadIdx.x; i < L.rows[X] * AH; i += ATHREADS) {
+            const int j = i / AH, src = param_row(X, out, j, P.M);
+            sw[L.w2[X] + j * WS + i % AH] = src >= 0 ? P.w2[X][src * AH + i % AH] : 0.f;
+        }
+        for (int j = threadIdx.x; j < L.rows[X]; j += ATHREADS) {
+            const int src = param_row(X, out, j, P.M);
+            sw[L.b2[X] + j] = src >= 0 ? P.b2[X][src] : 0.f;
+        }
     }
 }
 
-// h = relu(W1 f + b1); *mask gets bit k set where the pre-activation of
-// hidden unit k is positive.
+// A tile of TA = 32 RA anchors: arrays are [row][anchor], rows S floats
+// apart (16-byte aligned, and neighbouring rows start 4 banks apart).  Thread
+// tid owns anchors a0 .. a0 + RA - 1 of a group of 4 rows; a warp covers 8
+// anchor groups x 4 row groups.
+template <int RA>
+struct Tile {
+    static constexpr int TA = 32 * RA, S = TA + 4;
+    __device__ static __forceinline__ int anchor(int tid) {
+        return ((tid & 7) + 8 * ((tid >> 5) & 3)) * RA;
+    }
+    __device__ static __forceinline__ int group(int tid) {
+        return ((tid >> 3) & 3) + 4 * (tid >> 7);
+    }
+};
+constexpr int GROUPS = ATHREADS / 32;  // row groups of a block
+
+template <int RA>
+__device__ __forceinline__ void ld_anchors(const float* p, float (&v)[RA]) {
+    if constexpr (RA == 4) {
+        const float4 q = *reinterpret_cast<const float4*>(p);
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+    } else if constexpr (RA == 2) {
+        const float2 q = *reinterpret_cast<const float2*>(p);
+        v[0] = q.x; v[1] = q.y;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int RA>
+__device__ __forceinline__ void st_anchors(float* p, const float (&v)[RA]) {
+    if constexpr (RA == 4)
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (RA == 2)
+        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    else
+        *p = v[0];
+}
+
+// acc[r][a] = b[r] + sum_k w[r][k] x[k][a] over 32 inputs k in order, for 4
+// rows of weights (WS apart) and RA anchors of the tile x.
+template <int RA>
+__device__ __forceinline__ void tile_rows(const float* w, const float* b, const float* x,
+                                          float (&acc)[4][RA]) {
+    constexpr int S = Tile<RA>::S;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int a = 0; a < RA; ++a) acc[r][a] = b[r];
+#pragma unroll 2
+    for (int k = 0; k < 32; k += 4) {
+        float wv[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float4 q = *reinterpret_cast<const float4*>(w + r * WS + k);
+            wv[r][0] = q.x; wv[r][1] = q.y; wv[r][2] = q.z; wv[r][3] = q.w;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            float xv[RA];
+            ld_anchors<RA>(x + (k + e) * S, xv);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int a = 0; a < RA; ++a) acc[r][a] = fmaf(wv[r][e], xv[a], acc[r][a]);
+        }
+    }
+}
+
+// acc[c][a] += sum_j w[j][c] x[j][a] over n rows j in order, for 4 columns of
+// the weights.
+template <int RA>
+__device__ __forceinline__ void tile_cols(const float* w, const float* x, int n,
+                                          float (&acc)[4][RA]) {
+    constexpr int S = Tile<RA>::S;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+        const float4 q = *reinterpret_cast<const float4*>(w + j * WS);
+        const float wv[4] = {q.x, q.y, q.z, q.w};
+        float xv[RA];
+        ld_anchors<RA>(x + j * S, xv);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int a = 0; a < RA; ++a) acc[c][a] = fmaf(wv[c], xv[a], acc[c][a]);
+    }
+}
+
+// Features of the tile's anchors, transposed (zero past the last anchor).
+template <int RA>
+__device__ __forceinline__ void load_feat(const AnchorIn& P, int64_t base, int rows, float* ft) {
+    using T = Tile<RA>;
+    for (int i = threadIdx.x; i < T::TA * (AF / 4); i += ATHREADS) {
+        const int a = i / (AF / 4), q = i % (AF / 4);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (a < rows) v = reinterpret_cast<const float4*>(P.feat + (base + a) * AF)[q];
+        float* dst = ft + 4 * q * T::S + a;
+        dst[0] = v.x;
+        dst[T::S] = v.y;
+        dst[2 * T::S] = v.z;
+        dst[3 * T::S] = v.w;
+    }
+}
+
+// h = relu(W1 f + b1) of branch X for the tile.
+template <int RA>
 __device__ __forceinline__ void hidden_layer(const float* sw, const WLayout& L, int X,
-                                             const float (&f)[AF], float (&h)[AH],
-                                             uint32_t* mask) {
-    const float* w1 = sw + L.w1[X];
-    const float* b1 = sw + L.b1[X];
-    uint32_t m = 0u;
+                                             const float* ft, float* h) {
+    using T = Tile<RA>;
+    const int a0 = T::anchor(threadIdx.x), k0 = 4 * T::group(threadIdx.x);
+    float acc[4][RA];
+    tile_rows<RA>(sw + L.w1[X] + k0 * WS, sw + L.b1[X] + k0, ft + a0, acc);
 #pragma unroll
-    for (int k = 0; k < AH; ++k) {
-        float acc = b1[k];
+    for (int r = 0; r < 4; ++r) {
 #pragma unroll
-        for (int i = 0; i < AF; ++i) acc = fmaf(w1[k * AF + i], f[i], acc);
-        h[k] = fmaxf(acc, 0.f);
-        m |= (acc > 0.f ? 1u : 0u) << k;
-    }
-    *mask = m;
-}
-
-// Output j of MLP X: (W2 h + b2)_j.
-__device__ __forceinline__ float mlp_out(const float* sw, const WLayout& L, int X,
-                                         const float (&h)[AH], int j) {
-    const float* w2 = sw + L.w2[X] + j * AH;
-    float acc = sw[L.b2[X] + j];
-#pragma unroll
-    for (int k = 0; k < AH; ++k) acc = fmaf(w2[k], h[k], acc);
-    return acc;
-}
-
-__device__ __forceinline__ void load_feat(const AnchorIn& P, int64_t a, float (&f)[AF]) {
-    const float4* src = reinterpret_cast<const float4*>(P.feat + a * AF);
-#pragma unroll
-    for (int q = 0; q < AF / 4; ++q) {
-        const float4 v = src[q];
-        f[4 * q] = v.x;
-        f[4 * q + 1] = v.y;
-        f[4 * q + 2] = v.z;
-        f[4 * q + 3] = v.w;
+        for (int a = 0; a < RA; ++a) acc[r][a] = fmaxf(acc[r][a], 0.f);
+        st_anchors<RA>(h + (k0 + r) * T::S + a0, acc[r]);
     }
 }
 
-// The five branches run in a loop that is not unrolled, so the kernel holds
-// one copy of the fully unrolled 32 x 32 hidden layer (five copies made the
-// translation unit take minutes to compile).
+// Rows of the output buffer: the widest branch, padded.
+__host__ __device__ inline int out_rows(const WLayout& L) {
+    int m = 0;
+    for (int X = 0; X < NMLP; ++X) m = L.rows[X] > m ? L.rows[X] : m;
+    return m;
+}
+
+template <int RA>
+__host__ __device__ inline size_t decode_floats(const WLayout& L, int M) {
+    // the logits' rows are kept [anchor][channel]; the covariance branch's
+    // scales and quaternions take turns
+    const int sem = Tile<RA>::TA * (L.rows[0] + 4), y = 4 * M * Tile<RA>::S;
+    return (size_t)L.total + 2 * 32 * Tile<RA>::S + (sem > y ? sem : y);
+}
+
+template <int RA>
 __global__ void __launch_bounds__(ATHREADS) anchor_decode_kernel(const AnchorIn P, const WLayout L,
                                                                  const DecodeOut O, int bf16) {
+    using T = Tile<RA>;
+    constexpr int S = T::S;
     extern __shared__ __align__(16) float sw[];
+    float* ft = sw + L.total;  // [AF][S] features
+    float* h = ft + AF * S;    // [AH][S] hidden layer of one branch
+    float* y = h + AH * S;     // [rows][S] outputs of one branch
     load_weights(P, L, sw);
-    __syncthreads();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int M = P.M, C = P.C;
     const int64_t N = P.n * M;
     const bool fb = bf16 != 0;
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < P.n;
-         a += (int64_t)gridDim.x * blockDim.x) {
-        float f[AF], h[AH];
-        uint32_t mask;
-        load_feat(P, a, f);
-        const int64_t g0 = a * M;
-        const float l[3] = {P.scale[a], P.scale[P.n + a], P.scale[2 * P.n + a]};
+    const int a0 = T::anchor(tid), g0 = T::group(tid);
+    // whole 16-byte chunks of a Gaussian's logit row
+    const int cstr = L.rows[0] + 4;
+    const int row_bytes = C * (fb ? 2 : 4);
+    const bool vec = row_bytes % 16 == 0 && (reinterpret_cast<uintptr_t>(O.sem) & 15) == 0;
+    for (int64_t base = blockIdx.x * (int64_t)T::TA; base < P.n;
+         base += (int64_t)gridDim.x * T::TA) {
+        const int rows = (int)min((int64_t)T::TA, P.n - base);
+        const int kids = rows * M;      // Gaussians of the tile
+        const int64_t gb = base * M;    // the first of them
+        __syncthreads();
+        load_feat<RA>(P, base, rows, ft);
+        __syncthreads();
 #pragma unroll 1
-        for (int X = 0; X < NMLP; ++X) {
+        for (int step = 0; step <= NMLP; ++step) {
+            const int X = step < NMLP ? step : NMLP - 1;
             if (L.out[X] == 0) continue;  // no semantic branch without logits
-            hidden_layer(sw, L, X, f, h, &mask);
+            if (step != 5) {
+                hidden_layer<RA>(sw, L, X, ft, h);
+                __syncthreads();
+            }
+            // the quaternions (step 5) follow the scales in the same branch
+            const int jb = step == 5 ? quat_row(M) : 0;
+            const int je = step == 4 ? quat_row(M) : L.rows[X];
+#pragma unroll 1
+            for (int j0 = jb + 4 * g0; j0 < je; j0 += 4 * GROUPS) {
+                float acc[4][RA];
+                tile_rows<RA>(sw + L.w2[X] + j0 * WS, sw + L.b2[X] + j0, h + a0, acc);
+                if (X == 0) {
+                    // semantic logits: o_ah (x) sigma(MLP_sem(f)), the same for every child
+#pragma unroll
+                    for (int a = 0; a < RA; ++a)
+#pragma unroll
+                        for (int r = 0; r < 4; ++r)
+                            if (a0 + a < rows && j0 + r < C)
+                                y[(a0 + a) * cstr + j0 + r] =
+                                    P.sem[(base + a0 + a) * C + j0 + r] * sigm(acc[r][a]);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        st_anchors<RA>(y + (j0 - jb + r) * S + a0, acc[r]);
+                }
+            }
+            __syncthreads();
             if (X == 0) {
-                // semantic logits: o_ah (x) sigma(MLP_sem(f)), the same for every child
-                for (int c = 0; c < C; ++c) {
-                    const float o = P.sem[a * C + c] * sigm(mlp_out(sw, L, 0, h, c));
-                    for (int m = 0; m < M; ++m) put_feat(O.sem, (g0 + m) * C + c, o, fb);
+                // a warp per anchor: its M equal rows are one contiguous block
+                for (int a = warp; a < rows; a += ATHREADS / 32) {
+                    const float* src = y + a * cstr;
+                    const int64_t dst = (base + a) * M * C;
+                    if (vec && fb) {
+                        const int cpr = C / 8;
+                        uint4* d4 = reinterpret_cast<uint4*>(
+                            static_cast<__nv_bfloat16*>(O.sem) + dst);
+                        for (int i = lane; i < M * cpr; i += 32) {
+                            const float* s8 = src + (i % cpr) * 8;
+                            uint32_t q[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                q[e] = (uint32_t)__bfloat16_as_ushort(
+                                           __float2bfloat16_rn(s8[2 * e])) |
+                                       ((uint32_t)__bfloat16_as_ushort(
+                                            __float2bfloat16_rn(s8[2 * e + 1]))
+                                        << 16);
+                            d4[i] = make_uint4(q[0], q[1], q[2], q[3]);
+                        }
+                    } else if (vec) {
+                        const int cpr = C / 4;
+                        float4* d4 = reinterpret_cast<float4*>(static_cast<float*>(O.sem) + dst);
+                        for (int i = lane; i < M * cpr; i += 32)
+                            d4[i] = *reinterpret_cast<const float4*>(src + (i % cpr) * 4);
+                    } else {
+                        for (int i = lane; i < M * C; i += 32)
+                            put_feat(O.sem, dst + i, src[i % C], fb);
+                    }
                 }
             } else if (X == 1) {
                 // gradient factor: k_ah sigma(MLP_k(f))
-                const float k = P.kfac[a] * sigm(mlp_out(sw, L, 1, h, 0));
-                for (int m = 0; m < M; ++m) O.kfac[g0 + m] = k;
+                for (int i = tid; i < kids; i += ATHREADS) {
+                    const int a = i / M;
+                    O.kfac[gb + i] = P.kfac[base + a] * sigm(y[a]);
+                }
             } else if (X == 2) {
-                for (int m = 0; m < M; ++m) O.opacity[g0 + m] = sigm(mlp_out(sw, L, 2, h, m));
+                for (int i = tid; i < kids; i += ATHREADS)
+                    O.opacity[gb + i] = sigm(y[(i % M) * S + i / M]);
             } else if (X == 3) {
                 // colour as the degree-0 SH coefficient
-                for (int m = 0; m < M; ++m)
-                    for (int ch = 0; ch < 3; ++ch) {
-                        const float c = sigm(mlp_out(sw, L, 3, h, 3 * m + ch));
-                        put_feat(O.sh, (g0 + m) * 3 + ch, (c - 0.5f) / Y00, fb);
+                for (int i = tid; i < 3 * kids; i += ATHREADS) {
+                    const float c = sigm(y[(i % (3 * M)) * S + i / (3 * M)]);
+                    put_feat(O.sh, 3 * gb + i, (c - 0.5f) / Y00, fb);
+                }
+            } else if (step == 4) {
+                // scale, and the position x + l (x) O_m
+                for (int i = tid; i < kids; i += ATHREADS) {
+                    const int a = i / M, m = i % M;
+                    const int64_t g = gb + i;
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        const float l = P.scale[d * P.n + base + a];
+                        O.scale[d * N + g] = l * sigm(y[(3 * m + d) * S + a]);
+                        O.mean[d * N + g] = fmaf(l, P.offsets[g * 3 + d], P.pos[d * P.n + base + a]);
                     }
+                }
             } else {
-                // scale and rotation
-                for (int m = 0; m < M; ++m) {
-                    const int64_t g = g0 + m;
-                    for (int i = 0; i < 3; ++i)
-                        O.scale[i * N + g] = l[i] * sigm(mlp_out(sw, L, 4, h, 7 * m + i));
+                for (int i = tid; i < kids; i += ATHREADS) {
+                    const int a = i / M, m = i % M;
+#pragma unroll
                     for (int j = 0; j < 4; ++j)
-                        O.quat[j * N + g] = mlp_out(sw, L, 4, h, 7 * m + 3 + j);
+                        O.quat[j * N + gb + i] = y[(4 * m + j) * S + a];
                 }
             }
+            __syncthreads();
         }
-        // position: x + l (x) O_m
-        const float x[3] = {P.pos[a], P.pos[P.n + a], P.pos[2 * P.n + a]};
-        for (int m = 0; m < M; ++m)
-            for (int i = 0; i < 3; ++i)
-                O.mean[i * N + g0 + m] = fmaf(l[i], P.offsets[(g0 + m) * 3 + i], x[i]);
     }
 }
 
@@ -187,14 +379,9 @@ struct AnchorGradOut {
     int accumulate;
 };
 
-// Row strides (floats) of the shared-memory tiles: odd, so that the rows of
-// a warp's 32 threads start in 32 different banks.
-constexpr int GYS = MAXOUT + 1;
-constexpr int HS = AH + 1;
-constexpr int FS = AF + 1;
-
-__host__ __device__ constexpr size_t bwd_tile_floats() {
-    return (size_t)ATHREADS * (GYS + 2 * HS + FS);
+template <int RA>
+__host__ __device__ inline size_t bwd_floats(const WLayout& L, int M) {
+    return 2 * (size_t)L.total + (size_t)Tile<RA>::S * (3 * 32 + out_rows(L) + 3 * M);
 }
 
 __device__ __forceinline__ float gin(const float* p, int64_t i) { return p ? p[i] : 0.f; }
@@ -205,163 +392,216 @@ __device__ __forceinline__ void put(float* p, int64_t i, float v, int acc) {
         p[i] = v;
 }
 
+// s[i][j] += sum over the tile's anchors (in order) of x[i][a] z[j][a], 4 x 4
+// entries; with `bias` also b[i] += sum_a x[i][a].
+template <int RA>
+__device__ __forceinline__ void outer_sums(const float* x, const float* z, float* s, float* b,
+                                           bool bias) {
+    using T = Tile<RA>;
+    float acc[4][4] = {}, sb[4] = {};
+    for (int a = 0; a < T::TA; a += 4) {
+        float xv[4][4], zv[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            ld_anchors<4>(x + r * T::S + a, xv[r]);
+            ld_anchors<4>(z + r * T::S + a, zv[r]);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (bias) sb[i] += xv[i][e];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xv[i][e], zv[j][e], acc[i][j]);
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float4* d = reinterpret_cast<float4*>(s + i * WS);
+        float4 q = *d;
+        q.x += acc[i][0]; q.y += acc[i][1]; q.z += acc[i][2]; q.w += acc[i][3];
+        *d = q;
+        if (bias) b[i] += sb[i];
+    }
+}
+
+template <int RA>
 __global__ void __launch_bounds__(ATHREADS) anchor_decode_bwd_kernel(const AnchorIn P,
                                                                      const WLayout L,
                                                                      const GradIn G,
                                                                      const AnchorGradOut R) {
+    using T = Tile<RA>;
+    constexpr int S = T::S;
     extern __shared__ __align__(16) float sm[];
-    float* sw = sm;                     // parameters
-    float* sg = sw + L.total;           // parameter gradients of this block
-    float* gy = sg + L.total;           // [ATHREADS][GYS] output gradients of one branch
-    float* hid = gy + ATHREADS * GYS;   // [ATHREADS][HS] hidden activations
-    float* gpre = hid + ATHREADS * HS;  // [ATHREADS][HS] pre-activation gradients
-    float* ft = gpre + ATHREADS * HS;   // [ATHREADS][FS] features
+    float* sw = sm;               // parameters
+    float* sg = sw + L.total;     // parameter gradients of this block, same layout
+    float* ft = sg + L.total;     // [AF][S] features
+    float* h = ft + AF * S;       // [AH][S] hidden layer of one branch
+    float* gp = h + AH * S;       // [AH][S] its pre-activation gradients
+    float* sv = gp + AH * S;      // [3 M][S] sigma of the scale outputs
+    float* gy = sv + 3 * P.M * S; // [rows][S] output gradients of one branch
     load_weights(P, L, sw);
-    for (int i = threadIdx.x; i < L.total; i += blockDim.x) sg[i] = 0.f;
-    __syncthreads();
-    const int tid = threadIdx.x, M = P.M, C = P.C, acc = R.accumulate;
+    for (int i = threadIdx.x; i < L.total; i += ATHREADS) sg[i] = 0.f;
+    const int tid = threadIdx.x, M = P.M, C = P.C, acc_out = R.accumulate;
     const int64_t N = P.n * M;
-    for (int64_t base = blockIdx.x * (int64_t)ATHREADS; base < P.n;
-         base += (int64_t)gridDim.x * ATHREADS) {
-        const int64_t a = base + tid;
-        const bool valid = a < P.n;
-        const int rows = (int)min((int64_t)ATHREADS, P.n - base);
-        const int64_t g0 = a * M;
-        float f[AF], gf[AF];
-        if (valid)
-            load_feat(P, a, f);
-        else
+    const int a0 = T::anchor(tid), g0 = T::group(tid);
+    const bool vec = C % 4 == 0 && (reinterpret_cast<uintptr_t>(G.sem) & 15) == 0;
+    for (int64_t base = blockIdx.x * (int64_t)T::TA; base < P.n;
+         base += (int64_t)gridDim.x * T::TA) {
+        const int rows = (int)min((int64_t)T::TA, P.n - base);
+        __syncthreads();
+        load_feat<RA>(P, base, rows, ft);
+        float gf[4][RA];  // dL/df of features 4 g0 .. 4 g0 + 3
 #pragma unroll
-            for (int i = 0; i < AF; ++i) f[i] = 0.f;
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int i = 0; i < AF; ++i) {
-            ft[tid * FS + i] = f[i];
-            gf[i] = 0.f;
-        }
-        float l[3] = {0.f, 0.f, 0.f}, gl[3] = {0.f, 0.f, 0.f};
-        if (valid)
-            for (int i = 0; i < 3; ++i) l[i] = P.scale[i * P.n + a];
-        float* gyr = gy + tid * GYS;
+            for (int a = 0; a < RA; ++a) gf[r][a] = 0.f;
+        __syncthreads();
+#pragma unroll 1
         for (int X = 0; X < NMLP; ++X) {
-            const int out = L.out[X];
+            const int out = L.out[X], nr = L.rows[X];
             if (out == 0) continue;  // uniform: no semantic branch without logits
-            float h[AH];
-            uint32_t mask;
-            hidden_layer(sw, L, X, f, h, &mask);
-            // dL/d(branch output)
-            if (!valid) {
-                for (int j = 0; j < out; ++j) gyr[j] = 0.f;
-            } else if (X == 0) {
-                for (int c = 0; c < C; ++c) {
-                    const float s = sigm(mlp_out(sw, L, 0, h, c));
-                    float gc = 0.f;
-                    for (int m = 0; m < M; ++m) gc += gin(G.sem, (g0 + m) * C + c);
-                    put(R.sem, a * C + c, gc * s, acc);
-                    gyr[c] = gc * P.sem[a * C + c] * s * (1.f - s);
-                }
-            } else if (X == 1) {
-                const float s = sigm(mlp_out(sw, L, 1, h, 0));
-                float gk = 0.f;
-                for (int m = 0; m < M; ++m) gk += gin(G.kfac, g0 + m);
-                put(R.kfac, a, gk * s, acc);
-                gyr[0] = gk * P.kfac[a] * s * (1.f - s);
-            } else if (X == 2) {
-                for (int m = 0; m < M; ++m) {
-                    const float s = sigm(mlp_out(sw, L, 2, h, m));
-                    gyr[m] = gin(G.opacity, g0 + m) * s * (1.f - s);
-                }
-            } else if (X == 3) {
-                for (int j = 0; j < 3 * M; ++j) {
-                    const float c = sigm(mlp_out(sw, L, 3, h, j));
-                    gyr[j] = gin(G.sh, g0 * 3 + j) / Y00 * c * (1.f - c);
-                }
-            } else {
-                for (int m = 0; m < M; ++m) {
-                    const int64_t g = g0 + m;
-                    for (int i = 0; i < 3; ++i) {
-                        const float s = sigm(mlp_out(sw, L, 4, h, 7 * m + i));
-                        const float gs = gin(G.scale, i * N + g);
-                        gyr[7 * m + i] = gs * l[i] * s * (1.f - s);
-                        gl[i] = fmaf(gs, s, gl[i]);
+            hidden_layer<RA>(sw, L, X, ft, h);
+            __syncthreads();
+            // dL/d(branch output); the quaternions' outputs are linear and are
+            // not needed themselves
+            const int ny = X == 4 ? quat_row(M) : nr;
+#pragma unroll 1
+            for (int j0 = 4 * g0; j0 < ny; j0 += 4 * GROUPS) {
+                float yv[4][RA], gv[4][RA];
+                tile_rows<RA>(sw + L.w2[X] + j0 * WS, sw + L.b2[X] + j0, h + a0, yv);
+#pragma unroll
+                for (int a = 0; a < RA; ++a) {
+                    const bool ok = a0 + a < rows;
+                    const int64_t ga = base + a0 + a;  // anchor
+                    float u[4] = {0.f, 0.f, 0.f, 0.f};
+                    if (X == 0 && ok && G.sem) {
+                        const float* src = G.sem + ga * M * C + j0;
+                        if (vec) {
+#pragma unroll 4
+                            for (int m = 0; m < M; ++m) {
+                                const float4 q = *reinterpret_cast<const float4*>(src + m * C);
+                                u[0] += q.x; u[1] += q.y; u[2] += q.z; u[3] += q.w;
+                            }
+                        } else {
+                            for (int m = 0; m < M; ++m)
+#pragma unroll
+                                for (int r = 0; r < 4; ++r)
+                                    if (j0 + r < C) u[r] += src[m * C + r];
+                        }
                     }
-                    for (int j = 0; j < 4; ++j) gyr[7 * m + 3 + j] = gin(G.quat, j * N + g);
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int j = j0 + r;
+                        float v = 0.f;
+                        if (ok && j < (X == 4 ? 3 * M : out)) {
+                            const float s = sigm(yv[r][a]);
+                            if (X == 0) {
+                                put(R.sem, ga * C + j, u[r] * s, acc_out);
+                                v = u[r] * P.sem[ga * C + j] * s * (1.f - s);
+                            } else if (X == 1) {
+                                float gk = 0.f;
+                                for (int m = 0; m < M; ++m) gk += gin(G.kfac, ga * M + m);
+                                put(R.kfac, ga, gk * s, acc_out);
+                                v = gk * P.kfac[ga] * s * (1.f - s);
+                            } else if (X == 2) {
+                                v = gin(G.opacity, ga * M + j) * s * (1.f - s);
+                            } else if (X == 3) {
+                                v = gin(G.sh, ga * M * 3 + j) / Y00 * s * (1.f - s);
+                            } else {
+                                const int d = j % 3;
+                                v = gin(G.scale, d * N + ga * M + j / 3) *
+                                    P.scale[d * P.n + ga] * s * (1.f - s);
+                                sv[j * S + a0 + a] = s;
+                            }
+                        }
+                        gv[r][a] = v;
+                    }
                 }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) st_anchors<RA>(gy + (j0 + r) * S + a0, gv[r]);
             }
-#pragma unroll
-            for (int k = 0; k < AH; ++k) hid[tid * HS + k] = h[k];
-            // back through the branch: dL/dh = W2^T gy, the relu, dL/df += W1^T gpre
-            float gh[AH];
-#pragma unroll
-            for (int k = 0; k < AH; ++k) gh[k] = 0.f;
-            for (int j = 0; j < out; ++j) {
-                const float v = gyr[j];
-                const float* w2 = sw + L.w2[X] + j * AH;
-#pragma unroll
-                for (int k = 0; k < AH; ++k) gh[k] = fmaf(w2[k], v, gh[k]);
-            }
-            const float* w1 = sw + L.w1[X];
-#pragma unroll
-            for (int k = 0; k < AH; ++k) {
-                const float gp = ((mask >> k) & 1u) ? gh[k] : 0.f;
-                gpre[tid * HS + k] = gp;
-#pragma unroll
-                for (int i = 0; i < AF; ++i) gf[i] = fmaf(w1[k * AF + i], gp, gf[i]);
+            if (X == 4) {
+                for (int i = tid; i < 4 * T::TA * M; i += ATHREADS) {
+                    // Gaussian g of the tile, quaternion component d
+                    const int d = i / (T::TA * M), g = i % (T::TA * M);
+                    gy[(quat_row(M) + 4 * (g % M) + d) * S + g / M] =
+                        g < rows * M ? gin(G.quat, d * N + base * M + g) : 0.f;
+                }
             }
             __syncthreads();
-            // parameter gradients over the block's anchors; every entry has a
-            // fixed owner thread, so the shared accumulators need no atomics
-            for (int e = tid; e < out * AH; e += ATHREADS) {
-                const int j = e / AH, k = e % AH;
-                float s = 0.f;
-                for (int r = 0; r < rows; ++r) s = fmaf(gy[r * GYS + j], hid[r * HS + k], s);
-                sg[L.w2[X] + e] += s;
+            // back through the branch: dL/dh = W2^T gy, the relu
+            {
+                float gh[4][RA] = {};
+                tile_cols<RA>(sw + L.w2[X] + 4 * g0, gy + a0, nr, gh);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    float hv[RA];
+                    ld_anchors<RA>(h + (4 * g0 + r) * S + a0, hv);
+#pragma unroll
+                    for (int a = 0; a < RA; ++a) gh[r][a] = hv[a] > 0.f ? gh[r][a] : 0.f;
+                    st_anchors<RA>(gp + (4 * g0 + r) * S + a0, gh[r]);
+                }
             }
-            for (int j = tid; j < out; j += ATHREADS) {
-                float s = 0.f;
-                for (int r = 0; r < rows; ++r) s += gy[r * GYS + j];
-                sg[L.b2[X] + j] += s;
-            }
-            for (int e = tid; e < AH * AF; e += ATHREADS) {
-                const int k = e / AF, i = e % AF;
-                float s = 0.f;
-                for (int r = 0; r < rows; ++r) s = fmaf(gpre[r * HS + k], ft[r * FS + i], s);
-                sg[L.w1[X] + e] += s;
-            }
-            for (int k = tid; k < AH; k += ATHREADS) {
-                float s = 0.f;
-                for (int r = 0; r < rows; ++r) s += gpre[r * HS + k];
-                sg[L.b1[X] + k] += s;
+            __syncthreads();
+            // dL/df += W1^T gpre, and the parameter gradients over the tile's
+            // anchors; every entry has a fixed owner thread, so the shared
+            // accumulators need no atomics
+            tile_cols<RA>(sw + L.w1[X] + 4 * g0, gp + a0, AH, gf);
+            for (int t = tid; t < 64 + 2 * nr; t += ATHREADS) {
+                if (t < 64) {
+                    const int k = 4 * (t >> 3), i = 4 * (t & 7);
+                    outer_sums<RA>(gp + k * S, ft + i * S, sg + L.w1[X] + k * WS + i,
+                                   sg + L.b1[X] + k, i == 0);
+                } else {
+                    const int j = 4 * ((t - 64) >> 3), k = 4 * (t & 7);
+                    outer_sums<RA>(gy + j * S, h + k * S, sg + L.w2[X] + j * WS + k,
+                                   sg + L.b2[X] + j, k == 0);
+                }
             }
             __syncthreads();
         }
-        if (valid) {
-            // position and offsets: mu_m = x + l (x) O_m
-            float gx[3] = {0.f, 0.f, 0.f};
-            for (int m = 0; m < M; ++m)
-                for (int i = 0; i < 3; ++i) {
-                    const float gm = gin(G.mean, i * N + g0 + m);
-                    gx[i] += gm;
-                    gl[i] = fmaf(gm, P.offsets[(g0 + m) * 3 + i], gl[i]);
-                    put(R.offsets, (g0 + m) * 3 + i, gm * l[i], acc);
-                }
-            for (int i = 0; i < 3; ++i) {
-                put(R.pos, i * P.n + a, gx[i], acc);
-                put(R.scale, i * P.n + a, gl[i], acc);
-            }
+        // features, position, offsets and scale: mu_m = x + l (x) O_m
 #pragma unroll
-            for (int i = 0; i < AF; ++i) put(R.feat, a * AF + i, gf[i], acc);
+        for (int a = 0; a < RA; ++a)
+            if (a0 + a < rows)
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    put(R.feat, (base + a0 + a) * AF + 4 * g0 + r, gf[r][a], acc_out);
+        for (int i = tid; i < 3 * rows; i += ATHREADS) {
+            const int d = i / rows, a = i % rows;
+            const int64_t ga = base + a;
+            float gl = 0.f, gx = 0.f;
+            for (int m = 0; m < M; ++m)
+                gl = fmaf(gin(G.scale, d * N + ga * M + m), sv[(3 * m + d) * S + a], gl);
+            for (int m = 0; m < M; ++m) {
+                const float gm = gin(G.mean, d * N + ga * M + m);
+                gx += gm;
+                gl = fmaf(gm, P.offsets[(ga * M + m) * 3 + d], gl);
+            }
+            put(R.pos, d * P.n + ga, gx, acc_out);
+            put(R.scale, d * P.n + ga, gl, acc_out);
+        }
+        for (int i = tid; i < rows * M; i += ATHREADS) {
+            const int64_t g = base * M + i, ga = base + i / M;
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                put(R.offsets, g * 3 + d, gin(G.mean, d * N + g) * P.scale[d * P.n + ga], acc_out);
         }
     }
+    __syncthreads();
     // one atomic per parameter and block (cleared by the host without accumulate)
     for (int X = 0; X < NMLP; ++X) {
         if (L.out[X] == 0) continue;
-        for (int i = threadIdx.x; i < AH * AF; i += blockDim.x)
-            atomicAdd(R.w1[X] + i, sg[L.w1[X] + i]);
-        for (int i = threadIdx.x; i < AH; i += blockDim.x) atomicAdd(R.b1[X] + i, sg[L.b1[X] + i]);
-        for (int i = threadIdx.x; i < L.out[X] * AH; i += blockDim.x)
-            atomicAdd(R.w2[X] + i, sg[L.w2[X] + i]);
-        for (int i = threadIdx.x; i < L.out[X]; i += blockDim.x)
-            atomicAdd(R.b2[X] + i, sg[L.b2[X] + i]);
+        for (int i = tid; i < AH * AF; i += ATHREADS)
+            atomicAdd(R.w1[X] + i, sg[L.w1[X] + i / AF * WS + i % AF]);
+        for (int i = tid; i < AH; i += ATHREADS) atomicAdd(R.b1[X] + i, sg[L.b1[X] + i]);
+        for (int i = tid; i < L.rows[X] * AH; i += ATHREADS) {
+            const int j = i / AH, dst = param_row(X, L.out[X], j, M);
+            if (dst < 0) continue;
+            atomicAdd(R.w2[X] + dst * AH + i % AH, sg[L.w2[X] + j * WS + i % AH]);
+            if (i % AH == 0) atomicAdd(R.b2[X] + dst, sg[L.b2[X] + j]);
+        }
     }
 }
 
@@ -403,15 +643,16 @@ void make_layout(const unigs_anchors& a, unigs::WLayout& L, unigs::AnchorIn& P) 
         P.w2[X] = mlps[X]->w2;
         P.b2[X] = mlps[X]->b2;
         L.w1[X] = L.b1[X] = L.w2[X] = L.b2[X] = off;
+        L.rows[X] = X == 4 ? unigs::quat_row(M) + 4 * M : (outs[X] + 3) & ~3;
         if (outs[X] == 0) continue;
         L.w1[X] = off;
-        off += AH * AF;
+        off += AH * unigs::WS;
         L.b1[X] = off;
         off += AH;
         L.w2[X] = off;
-        off += outs[X] * AH;
+        off += L.rows[X] * unigs::WS;
         L.b2[X] = off;
-        off += outs[X];
+        off += L.rows[X];
     }
     L.total = off;
     P.n = a.n;
@@ -425,10 +666,24 @@ void make_layout(const unigs_anchors& a, unigs::WLayout& L, unigs::AnchorIn& P) 
     P.kfac = a.kfac;
 }
 
-int anchor_grid(int64_t n) {
-    const int64_t blocks = (n + unigs::ATHREADS - 1) / unigs::ATHREADS;
-    const int64_t cap = (int64_t)unigs::sm_count() * 8;
-    return (int)(blocks < cap ? blocks : cap);
+// Shared memory a block can have (sm_103a).
+constexpr size_t MAX_SMEM = 232448;
+
+// Anchors per tile / 32: 4 where that leaves every SM a tile and the buffers
+// fit, else 1, so that small sets still spread over the chip (a tile of 128
+// takes about three times as long as one of 32).
+bool wide_tiles(int64_t n, size_t floats) {
+    return n >= (int64_t)unigs::sm_count() * 128 && floats * sizeof(float) <= MAX_SMEM;
+}
+
+template <typename K, typename... Args>
+void launch_tiles(K kernel, int ta, size_t floats, int blocks_per_sm, int64_t n, cudaStream_t st,
+                  const Args&... args) {
+    const size_t smem = floats * sizeof(float);
+    const int64_t tiles = (n + ta - 1) / ta;
+    const int64_t cap = (int64_t)unigs::sm_count() * blocks_per_sm;
+    unigs::ensure_smem_limit(reinterpret_cast<const void*>(kernel), (int)smem);
+    kernel<<<(int)(tiles < cap ? tiles : cap), unigs::ATHREADS, smem, st>>>(args...);
 }
 
 unigs_status launch_status() {
@@ -451,11 +706,14 @@ extern "C" unigs_status unigs_anchor_decode(const unigs_anchors* a,
     make_layout(*a, L, P);
     unigs::DecodeOut O{out->mean, out->quat, out->scale, out->opacity, out->kfac, out->sh,
                        out->sem};
-    const size_t smem = sizeof(float) * (size_t)L.total;
-    const int grid = anchor_grid(a->n);
     cudaStream_t st = (cudaStream_t)stream;
-    unigs::ensure_smem_limit(reinterpret_cast<const void*>(&unigs::anchor_decode_kernel), (int)smem);
-    unigs::anchor_decode_kernel<<<grid, unigs::ATHREADS, smem, st>>>(P, L, O, out->feat_dtype);
+    const size_t wide = unigs::decode_floats<4>(L, P.M), narrow = unigs::decode_floats<1>(L, P.M);
+    if (wide_tiles(a->n, wide))
+        launch_tiles(&unigs::anchor_decode_kernel<4>, 128, wide, 2, a->n, st, P, L, O,
+                     out->feat_dtype);
+    else
+        launch_tiles(&unigs::anchor_decode_kernel<1>, 32, narrow, 2, a->n, st, P, L, O,
+                     out->feat_dtype);
     return launch_status();
 }
 
@@ -495,11 +753,13 @@ extern "C" unigs_status unigs_anchor_decode_bwd(const unigs_anchors* a, const un
     }
     if (a->n == 0) return launch_status();
     unigs::GradIn G{g->mean, g->quat, g->scale, g->opacity, g->kfac, g->sh, g->sem};
-    const size_t smem = sizeof(float) * (2 * (size_t)L.total + unigs::bwd_tile_floats());
-    const int64_t blocks = (a->n + unigs::ATHREADS - 1) / unigs::ATHREADS;
-    const int grid = (int)(blocks < unigs::sm_count() ? blocks : unigs::sm_count());
-    unigs::ensure_smem_limit(reinterpret_cast<const void*>(&unigs::anchor_decode_bwd_kernel),
-                             (int)smem);
-    unigs::anchor_decode_bwd_kernel<<<grid, unigs::ATHREADS, smem, st>>>(P, L, G, R);
+    const size_t wide = unigs::bwd_floats<4>(L, P.M), mid = unigs::bwd_floats<2>(L, P.M),
+                 narrow = unigs::bwd_floats<1>(L, P.M);
+    if (wide_tiles(a->n, wide))
+        launch_tiles(&unigs::anchor_decode_bwd_kernel<4>, 128, wide, 1, a->n, st, P, L, G, R);
+    else if (wide_tiles(a->n, mid))
+        launch_tiles(&unigs::anchor_decode_bwd_kernel<2>, 64, mid, 1, a->n, st, P, L, G, R);
+    else
+        launch_tiles(&unigs::anchor_decode_bwd_kernel<1>, 32, narrow, 1, a->n, st, P, L, G, R);
     return launch_status();
 }
