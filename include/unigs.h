@@ -197,7 +197,7 @@ typedef struct {
     int64_t n_pixels;       /* all cameras */
     int32_t tile_offset[UNIGS_MAX_CAMS + 1];
     int64_t pixel_offset[UNIGS_MAX_CAMS + 1];
-    int32_t sort_passes;    /* 8-bit radix passes over the used key bits */
+    int32_t sort_passes;    /* 8-bit digits of the used (tile, depth) key bits */
     int32_t reserved;
     size_t ws_bytes;
     size_t off[20];         /* internal region offsets */
@@ -236,10 +236,11 @@ size_t unigs_workspace_bytes(const unigs_plan* plan);
 unigs_status unigs_preprocess(const unigs_plan* plan, const unigs_gaussians* g,
                               const unigs_camera* cams, void* ws, unigs_stream stream);
 
-/* Binning: exclusive scan of tiles touched, emission of (global tile << 32 |
- * depth bits) keys with the Gaussian index as value, stable LSD radix sort of
- * the used key bits, and per-tile [start, end) ranges.  Within a tile the
- * order is (centre depth, Gaussian index).  If n_instances_out is non-NULL the
+/* Binning: stable radix sort of the (camera, Gaussian) pairs with a kept tile
+ * by depth, emission of one (global tile, Gaussian index) instance per kept
+ * tile in that order, stable radix sort by tile, and per-tile [start, end)
+ * ranges.  Within a tile the order is (centre depth, Gaussian index), that of
+ * the key (global tile << 32 | depth bits).  If n_instances_out is non-NULL the
  * stream is synchronised and the instance total written there; if the total
  * exceeds plan->capacity the call returns UNIGS_ERR_CAPACITY (nothing is
  * written out of bounds; re-plan with at least that capacity).  With NULL it
@@ -340,8 +341,7 @@ const char* unigs_status_string(unigs_status s);
  * or a real-time loop in which a cudaMalloc may not run).
  *
  * Stable LSD radix sort of n (key, value) pairs by the low key_bits bits of
- * the key - the sort unigs_bin_sort runs on the tile|depth keys - but with its
- * scratch memory (one ping-pong buffer, digit histograms, scan partials, a
+ * the key, with its scratch memory (one ping-pong buffer, digit histograms, scan partials, a
  * status block) in a static device array of the library rather than in a
  * caller workspace.  The caller passes device inputs and outputs only.
  * Sorted order: ascending (key mod 2^key_bits), ties in input order; key

@@ -1,17 +1,34 @@
-// Binning: scan of tiles touched, key emission, stable LSD radix sort, ranges.
+// Binning: a depth order of the kept pairs, emission, a stable sort by tile,
+// ranges; and the 64-bit pair sort of unigs_sort_pairs_static.
 //
 // The paper extends the tile pipeline of 3DGS (Sec. 3.4): each Gaussian is
 // duplicated once per tile its 3-sigma rectangle overlaps, keyed by
 // (global tile id << 32 | float32 bits of its camera-frame centre depth), and
-// the keys are sorted so that every tile holds a front-to-back list.  Depths
-// are > z_near > 0, so their bit patterns order like the values.  The sort is
-// a stable LSD radix sort over the used key bits (8-bit digits), so ties in
-// depth keep the emission order (Gaussian index): the order within a tile is
-// (depth, index).
+// sorted so that every tile holds a front-to-back list, ties in depth in
+// Gaussian order.  Sorting the instances by the whole key moves every one of
+// them once per digit of 32 + tile bits.  Here the (camera, Gaussian) pairs
+// with a kept tile, several times fewer than their instances, are sorted by
+// depth first (four 8-bit passes, stable from pair order; depths are
+// > z_near > 0, so their bit patterns order like the values).  The instances
+// are then emitted in that order, and a stable sort by tile id alone (digits
+// of at most 9 bits: one or two passes, 4-byte keys) leaves the same list.
 //
-// Every kernel reads the instance count from the workspace header, so the
-// whole sequence runs without a host round trip (CUDA-graph capture); grids
-// are sized from the plan's capacity and surplus blocks exit at once.
+// Each pass is one kernel: blocks take chunks by ticket, rank their keys in
+// shared memory, and find the global position of each digit by looking back
+// over the chunks before them (each chunk publishes its digit counts, then
+// its inclusive prefixes).  A chunk only waits for chunks whose ticket was
+// drawn earlier, so the wait ends; it is bounded all the same.
+//
+// Every kernel reads the instance count from device memory, so the whole
+// sequence runs without a host round trip (CUDA-graph capture).
+//
+// What bounds it: memory traffic on large inputs (a tile pass of 142M
+// instances moves 16 bytes each at 2.6 TB/s), launches on small ones.  Against
+// six or seven passes over 12-byte (key, value) pairs, each of a histogram, a
+// three-kernel scan and a scatter (31 to 36 launches instead of 10 to 12):
+// 16 views of 3M Gaussians, 142M instances, scan to ranges 13.3 -> 5.2 ms; one
+// 1280x720 view of 1M, 2.7M instances, 0.36 -> 0.22 ms; one 256x256 view of
+// 10k, 0.33 -> 0.24 ms for the whole frame.
 #include "launch.h"
 
 namespace unigs {
@@ -110,107 +127,535 @@ int scan_u32(const uint32_t* in, int64_t n, uint32_t* partial, uint32_t* out, ui
     return 3;
 }
 
-// ------------------------------------------------------------ emission
-// Total = offsets[last] + touched[last]; checks the capacity and writes one
-// (key, value) per overlapped tile in (camera, Gaussian, tile row-major)
-// order.
-__global__ void __launch_bounds__(256)
-    emit_kernel(const CamTable* __restrict__ tab, int64_t n, int n_cams, int tw, int th,
-                int64_t capacity,
-                const uint2* __restrict__ rect, const uint32_t* __restrict__ touched,
-                const uint32_t* __restrict__ offs, const uint32_t* __restrict__ zbits,
-                const float* __restrict__ cull, WsHeader* __restrict__ hdr,
-                unsigned long long* __restrict__ keys, uint32_t* __restrict__ vals) {
-    const int64_t total = n * (int64_t)n_cams;
-    const uint64_t need = (uint64_t)offs[total - 1] + touched[total - 1];
-    if (need > (uint64_t)capacity) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            hdr->need = need;
-            hdr->n_instances = 0;
-            set_status(hdr, UNIGS_ERR_CAPACITY);
-        }
-        return;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        hdr->n_instances = (uint32_t)need;
-        hdr->need = need;
-    }
-    const int lane = threadIdx.x & 31;
-    const uint32_t lt_mask = (1u << lane) - 1u;
-    // uniform loop bound: whole warps iterate together, so rectangles larger
-    // than 32 tiles are emitted cooperatively (ballot compaction keeps the
-    // row-major order)
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < total;
-         base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = base + threadIdx.x;
-        const uint32_t cnt = t < total ? touched[t] : 0u;
-        int x0 = 0, x1 = 0, y0 = 0, y1 = 0, k = 0;
-        uint32_t g = 0, o = 0;
-        unsigned long long zb = 0, toff = 0;
-        int tiles_x = 0;
-        float cr[CULL_FLOATS] = {};
-        if (cnt) {
-            k = (int)(t / n);
-            g = (uint32_t)(t - (int64_t)k * n);
-            const DevCam& cam = tab->cam[k];
-            const uint2 r = rect[t];
-            x0 = r.x & 0xffff; x1 = r.x >> 16; y0 = r.y & 0xffff; y1 = r.y >> 16;
-            zb = zbits[t];
-            toff = (unsigned long long)cam.tile_off;
-            tiles_x = cam.tiles_x;
-            o = offs[t];
-            const float4* src = reinterpret_cast<const float4*>(cull + (size_t)t * CULL_FLOATS);
-            const float4 c0 = src[0], c1 = src[1];
-            cr[0] = c0.x; cr[1] = c0.y; cr[2] = c0.z; cr[3] = c0.w;
-            cr[4] = c1.x; cr[5] = c1.y; cr[6] = c1.z; cr[7] = c1.w;
-        }
-        const int nt = (x1 - x0) * (y1 - y0);
-        if (cnt && nt <= COOP_TILES) {
-            const uint32_t o_end = o + cnt;
-            for (int ty = y0; ty < y1; ++ty)
-                for (int tx = x0; tx < x1; ++tx) {
-                    if (!tile_keep(cr, tx, ty, tw, th) || o >= o_end) continue;
-                    const unsigned long long tile = toff + (unsigned long long)(ty * tiles_x + tx);
-                    keys[o] = (tile << 32) | zb;
-                    vals[o] = g;
-                    ++o;
-                }
-        }
-        unsigned big = __ballot_sync(0xffffffffu, cnt && nt > COOP_TILES);
-        while (big) {
-            const int src = __ffs(big) - 1;
-            big &= big - 1;
-            float cb[CULL_FLOATS];
+// ------------------------------------------------------- single-kernel passes
+// A look-back word: (epoch << 2 | state) << 32 | count.  state 1: the chunk's
+// own count, 2: its inclusive prefix; any other epoch: not written yet.
+__device__ __forceinline__ void lb_store(unsigned long long* w, uint32_t epoch, uint32_t state,
+                                         uint32_t count) {
+    const unsigned long long v = ((unsigned long long)(epoch << 2 | state) << 32) | count;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long lb_load(const unsigned long long* w) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(w) : "memory");
+    return v;
+}
+
+constexpr uint32_t LB_WAIT_LIMIT = 1u << 20;  // polls of one word, about a second
+constexpr int LB_WIDE = 8;                    // predecessors read per step
+
+// Sum of the counts of chunks [0, chunk) in column `col` of the look-back
+// table (rows of `stride` words).  Reads LB_WIDE predecessors at a time: one
+// memory latency per step, where one at a time a full first wave of chunks
+// would pay a latency per chunk.  Returns false when a wait gave up.
+__device__ __forceinline__ bool look_back(const unsigned long long* words, int64_t chunk,
+                                          int stride, int col, uint32_t epoch, uint32_t* sum_out) {
+    uint32_t sum = 0, polls = 0;
+    int64_t p = chunk - 1;
+    while (p >= 0) {
+        unsigned long long v[LB_WIDE];
 #pragma unroll
-            for (int q = 0; q < CULL_FLOATS; ++q) cb[q] = __shfl_sync(0xffffffffu, cr[q], src);
-            const int bx0 = __shfl_sync(0xffffffffu, x0, src);
-            const int by0 = __shfl_sync(0xffffffffu, y0, src);
-            const int bw = __shfl_sync(0xffffffffu, x1 - x0, src);
-            const int bn = __shfl_sync(0xffffffffu, nt, src);
-            const int btx = __shfl_sync(0xffffffffu, tiles_x, src);
-            const unsigned long long btoff = __shfl_sync(0xffffffffu, toff, src);
-            const unsigned long long bzb = __shfl_sync(0xffffffffu, zb, src);
-            const uint32_t bg = __shfl_sync(0xffffffffu, g, src);
-            uint32_t bo = __shfl_sync(0xffffffffu, o, src);
-            const uint32_t bend = bo + __shfl_sync(0xffffffffu, cnt, src);
-            for (int j0 = 0; j0 < bn; j0 += 32) {
-                const int j = j0 + lane;
-                const int tx = bx0 + j % bw, ty = by0 + j / bw;
-                const bool keep = j < bn && tile_keep(cb, tx, ty, tw, th);
-                const unsigned m = __ballot_sync(0xffffffffu, keep);
-                const uint32_t dst = bo + __popc(m & lt_mask);
-                if (keep && dst < bend) {
-                    const unsigned long long tile = btoff + (unsigned long long)(ty * btx + tx);
-                    keys[dst] = (tile << 32) | bzb;
-                    vals[dst] = bg;
-                }
-                bo += __popc(m);
+        for (int j = 0; j < LB_WIDE; ++j)
+            v[j] = p - j >= 0 ? lb_load(words + (p - j) * stride + col) : 0ull;
+        int used = 0;
+        bool open = true, found = false;
+#pragma unroll
+        for (int j = 0; j < LB_WIDE; ++j) {
+            const uint32_t tag = (uint32_t)(v[j] >> 32);
+            open = open && !found && p - j >= 0 && (tag >> 2) == epoch && (tag & 3u) != 0u;
+            if (open) {
+                sum += (uint32_t)v[j];
+                found = (tag & 3u) == 2u;
+                ++used;
             }
         }
+        if (found) break;
+        p -= used;
+        if (used == 0 && ++polls > LB_WAIT_LIMIT) return false;
+    }
+    *sum_out = sum;
+    return true;
+}
+
+// Digit counts of the depth keys of the pairs with a kept tile, for all four
+// passes at once; clears the look-back words of the depth passes and of the
+// emission, and the ranges.
+__global__ void __launch_bounds__(512)
+    depth_hist_kernel(const uint32_t* __restrict__ touched, const uint32_t* __restrict__ zbits,
+                      int64_t total, SortState* __restrict__ st,
+                      unsigned long long* __restrict__ words, int64_t n_words,
+                      unsigned long long* __restrict__ emit_words, int64_t n_emit_words,
+                      uint2* __restrict__ ranges, int64_t n_tiles) {
+    __shared__ uint32_t h[4][256];
+    for (int j = threadIdx.x; j < 4 * 256; j += blockDim.x) (&h[0][0])[j] = 0;
+    __syncthreads();
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < n_words; i += stride) words[i] = 0ull;
+    for (int64_t i = i0; i < n_emit_words; i += stride) emit_words[i] = 0ull;
+    for (int64_t i = i0; i < n_tiles; i += stride) ranges[i] = make_uint2(0u, 0u);
+    uint32_t kept = 0;
+    for (int64_t i = i0; i < total; i += stride) {
+        if (touched[i] == 0) continue;
+        const uint32_t z = zbits[i];
+        ++kept;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) atomicAdd(&h[p][(z >> (8 * p)) & 255u], 1u);
+    }
+    kept = __reduce_add_sync(0xffffffffu, kept);
+    if ((threadIdx.x & 31) == 0 && kept) atomicAdd(&st->n_kept, kept);
+    __syncthreads();
+    for (int j = threadIdx.x; j < 4 * 256; j += blockDim.x) {
+        const uint32_t c = (&h[0][0])[j];
+        if (c) atomicAdd(&st->dhist[0][0] + j, c);
     }
 }
 
+struct OnesweepParams {
+    const uint32_t* kin;   // keys (FROM_PAIRS: depth bits of every pair)
+    const uint32_t* vin;   // values (FROM_PAIRS: touched counts, the value is the index)
+    uint32_t* kout;
+    uint32_t* vout;
+    const uint32_t* hist;  // digit counts of this pass
+    unsigned long long* words;
+    uint32_t* ticket;
+    const uint32_t* n_ptr; // element count on the device (FROM_PAIRS: n_host)
+    int64_t n_host;
+    SortState* st;
+    WsHeader* hdr;
+    int shift, bits;       // digit (key >> shift) & (2^bits - 1), bits <= 9
+    uint32_t epoch;
+};
+
+template <int PER>
+struct OnesweepSmem {
+    uint32_t sk[RS_THREADS * PER];
+    uint32_t sv[RS_THREADS * PER];
+    uint16_t whist[RS_WARPS][RS_BINS];
+    uint32_t goff[RS_BINS];  // global position of the block's first key of a digit
+    uint32_t loff[RS_BINS];  // its position in the block's staging
+    uint32_t base[RS_BINS];  // global position of the digit
+    uint32_t wsum[RS_WARPS];
+    uint32_t chunk;
+};
+
+// Exclusive scan over RS_THREADS values, one per thread.
+__device__ __forceinline__ uint32_t scan512(uint32_t v, uint32_t* wsum, uint32_t* total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[w] = x;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int i = 0; i < RS_WARPS; ++i) {
+        const uint32_t s = wsum[i];
+        if (i < w) before += s;
+        all += s;
+    }
+    __syncthreads();
+    *total = all;
+    return before + x - v;
+}
+
+// One stable radix pass.  Warp w of a block owns 32 PER consecutive keys of
+// the block's chunk and walks them 32 at a time in order: __match_any_sync
+// ranks equal digits inside a step, a running count per warp orders the
+// steps, a prefix over the warps orders the warps.  The pairs are placed in
+// shared memory in (digit, input) order and written out by consecutive
+// threads, so the pairs of a digit land at consecutive addresses.
+// FROM_PAIRS: the first depth pass, reading (touched, depth) of every
+// (camera, Gaussian) pair in pair order and dropping those without a kept
+// tile.  KEYS: also write the keys (the last depth pass needs only the order).
+template <int PER, bool FROM_PAIRS, bool KEYS>
+__global__ void __launch_bounds__(RS_THREADS, 2) onesweep_kernel(const OnesweepParams P) {
+    extern __shared__ __align__(16) unsigned char rs_raw[];
+    OnesweepSmem<PER>& S = *reinterpret_cast<OnesweepSmem<PER>*>(rs_raw);
+    constexpr int ITEMS = RS_THREADS * PER;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    const int bins = 1 << P.bits;
+    const uint32_t dmask = (uint32_t)bins - 1u;
+    const int64_t n = FROM_PAIRS ? P.n_host : (int64_t)*P.n_ptr;
+    uint32_t tot;
+    {
+        const uint32_t e = scan512(tid < bins ? P.hist[tid] : 0u, S.wsum, &tot);
+        S.base[tid] = e;
+    }
+    for (;;) {
+        // an earlier wait that gave up leaves nothing to sort (no such chunk)
+        if (tid == 0)
+            S.chunk = *(volatile uint32_t*)&P.st->abort ? ~0u : atomicAdd(P.ticket, 1u);
+        for (int j = tid; j < RS_WARPS * RS_BINS / 2; j += RS_THREADS)
+            reinterpret_cast<uint32_t*>(&S.whist[0][0])[j] = 0u;
+        __syncthreads();
+        const int64_t chunk = S.chunk;
+        const int64_t block0 = chunk * ITEMS;
+        if (block0 >= n) break;
+        const int64_t first = block0 + (int64_t)w * (32 * PER);
+        uint32_t k[PER], v[PER];
+        uint32_t rank[PER];  // digit << 16 | rank within the warp; ~0: no key
+#pragma unroll
+        for (int it = 0; it < PER; ++it) {
+            const int64_t i = first + it * 32 + lane;
+            bool ok = i < n;
+            k[it] = ok ? P.kin[i] : 0u;
+            v[it] = ok ? P.vin[i] : 0u;
+            if (FROM_PAIRS) {
+                ok = ok && v[it] != 0u;
+                v[it] = (uint32_t)i;
+            }
+            rank[it] = ok ? 0u : ~0u;
+        }
+#pragma unroll
+        for (int it = 0; it < PER; ++it) {
+            const bool ok = rank[it] == 0u;
+            const uint32_t d = ok ? (k[it] >> P.shift) & dmask : RS_BINS;
+            const uint32_t peers = __match_any_sync(0xffffffffu, d);
+            const uint32_t before = ok ? S.whist[w][d] : 0u;
+            __syncwarp();
+            if (ok && lane == __ffs(peers) - 1)
+                S.whist[w][d] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+            if (ok) rank[it] = (d << 16) | (before + __popc(peers & lt_mask));
+        }
+        __syncthreads();
+        // digit tid: its count, the warps' offsets within it, its staging offset
+        uint32_t cnt = 0;
+#pragma unroll
+        for (int w2 = 0; w2 < RS_WARPS; ++w2) {
+            const uint32_t c = S.whist[w2][tid];
+            S.whist[w2][tid] = (uint16_t)cnt;
+            cnt += c;
+        }
+        unsigned long long* row = P.words + chunk * bins + tid;
+        if (tid < bins) lb_store(row, P.epoch, chunk == 0 ? 2u : 1u, cnt);
+        const uint32_t lo = scan512(cnt, S.wsum, &tot);
+        S.loff[tid] = lo;
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < PER; ++it)
+            if (rank[it] != ~0u) {
+                const uint32_t d = rank[it] >> 16;
+                const uint32_t lp = S.loff[d] + S.whist[w][d] + (rank[it] & 0xffffu);
+                S.sk[lp] = k[it];
+                S.sv[lp] = v[it];
+            }
+        bool bad = false;
+        if (tid < bins) {
+            uint32_t before = 0;
+            if (chunk > 0) {
+                bad = !look_back(P.words, chunk, bins, tid, P.epoch, &before);
+                if (!bad) lb_store(row, P.epoch, 2u, before + cnt);
+            }
+            S.goff[tid] = S.base[tid] + before;
+        }
+        if (__syncthreads_or(bad)) {
+            if (tid == 0) {
+                atomicExch(&P.st->abort, 1u);
+                set_status(P.hdr, UNIGS_ERR_TIMEOUT);
+            }
+            break;
+        }
+        for (uint32_t j = tid; j < tot; j += RS_THREADS) {
+            const uint32_t key = S.sk[j];
+            const uint32_t d = (key >> P.shift) & dmask;
+            const uint32_t dst = S.goff[d] + (j - S.loff[d]);
+            if (KEYS) P.kout[dst] = key;
+            P.vout[dst] = S.sv[j];
+        }
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------ emission
+struct EmitParams {
+    const CamTable* tab;
+    int64_t n;
+    int tw, th;
+    int64_t capacity;
+    const uint2* rect;
+    const uint32_t* touched;
+    const unsigned long long* masks;
+    const float* cull;
+    const uint32_t* order;            // kept pairs by depth
+    SortState* st;
+    WsHeader* hdr;
+    unsigned long long* emit_words;   // look-back, one word per chunk
+    unsigned long long* words;        // look-back table of the tile passes, cleared here
+    uint4* big;                       // pairs left to emit_big_kernel
+    uint32_t* keys;                   // global tile ids
+    uint32_t* vals;                   // Gaussian indices
+    int passes, bits, items;          // tile passes: count, digit bits, keys per chunk
+};
+
+// Writes one instance and counts its tile digits.
+__device__ __forceinline__ void put_instance(const EmitParams& P, uint32_t (*hist)[RS_BINS],
+                                             uint32_t dst, uint32_t tile, uint32_t g) {
+    P.keys[dst] = tile;
+    P.vals[dst] = g;
+    const uint32_t dmask = (1u << P.bits) - 1u;
+    for (int p = 0; p < P.passes; ++p) atomicAdd(&hist[p][(tile >> (p * P.bits)) & dmask], 1u);
+}
+
+// The block's digit counts, added to the binning's.
+__device__ __forceinline__ void flush_hist(const EmitParams& P, uint32_t (*hist)[RS_BINS]) {
+    __syncthreads();
+    for (int p = 0; p < P.passes; ++p)
+        for (int j = threadIdx.x; j < (1 << P.bits); j += blockDim.x)
+            if (hist[p][j]) atomicAdd(&P.st->thist[p][j], hist[p][j]);
+}
+
+// Position of set bit number r of m (r < popcount(m)).
+__device__ __forceinline__ int nth_bit(unsigned long long m, int r) {
+    int pos = 0;
+    uint32_t x = (uint32_t)m;
+    int c = __popc(x);
+    if (r >= c) { r -= c; x = (uint32_t)(m >> 32); pos = 32; }
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        c = __popc(x & ((1u << s) - 1u));
+        if (r >= c) { r -= c; x >>= s; pos += s; }
+    }
+    return pos;
+}
+
+// One instance per kept tile, in (depth, pair) order.  A block takes 256
+// pairs, finds the position of its first instance by look-back, and its warps
+// write theirs from the preprocess's bit masks, one output slot per lane (so
+// that a warp's stores are consecutive whatever the rectangles' sizes).
+// Rectangles of more than MASK_TILES tiles are listed for emit_big_kernel:
+// in depth order the largest ones, those nearest the camera, all fall into the
+// first few blocks (emitted there, a 1280x720 view of 1M Gaussians took
+// 1.18 ms; with the list 0.034 + 0.051 ms).  Also counts the tile digits and clears the
+// look-back words of the chunks that its own instances start.
+__global__ void __launch_bounds__(256) emit_kernel(const EmitParams P) {
+    __shared__ uint32_t hist[TILE_PASSES_MAX][RS_BINS];
+    __shared__ uint32_t sw[32];
+    __shared__ uint32_t s_chunk;
+    __shared__ unsigned long long s_base;
+    __shared__ int s_bad;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int bins = 1 << P.bits;
+    for (int j = tid; j < P.passes * RS_BINS; j += 256) (&hist[0][0])[j] = 0u;
+    const int64_t n_kept = P.st->n_kept;
+    for (;;) {
+        if (tid == 0)
+            s_chunk = *(volatile uint32_t*)&P.st->abort ? ~0u
+                                                        : atomicAdd(&P.st->ticket[TICKET_EMIT], 1u);
+        __syncthreads();
+        const int64_t chunk = s_chunk;
+        if (chunk * 256 >= n_kept) break;
+        const int64_t i = chunk * 256 + tid;
+        uint32_t t = 0, cnt = 0;
+        if (i < n_kept) {
+            t = P.order[i];
+            cnt = P.touched[t];
+        }
+        uint32_t tot;
+        const uint32_t ex = block_exclusive_scan(cnt, sw, &tot);
+        // the instances of all chunks may exceed 32 bits (then far over the
+        // capacity): the words' 62-bit counts are kept apart from the state
+        // in the two top bits
+        if (tid == 0) {
+            constexpr unsigned long long VAL = (1ull << 62) - 1ull;
+            unsigned long long base = 0;
+            unsigned long long* w = P.emit_words;
+            int bad = 0;
+            const unsigned long long own = ((chunk == 0 ? 2ull : 1ull) << 62) | tot;
+            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w + chunk), "l"(own) : "memory");
+            uint32_t polls = 0;
+            for (int64_t p = chunk - 1; p >= 0;) {
+                unsigned long long v[LB_WIDE];
+#pragma unroll
+                for (int j = 0; j < LB_WIDE; ++j) v[j] = p - j >= 0 ? lb_load(w + p - j) : 0ull;
+                int used = 0;
+                bool open = true, found = false;
+#pragma unroll
+                for (int j = 0; j < LB_WIDE; ++j) {
+                    open = open && !found && (v[j] >> 62) != 0ull;
+                    if (open) {
+                        base += v[j] & VAL;
+                        found = (v[j] >> 62) == 2ull;
+                        ++used;
+                    }
+                }
+                if (found) break;
+                p -= used;
+                if (used == 0 && ++polls > LB_WAIT_LIMIT) {
+                    bad = 1;
+                    break;
+                }
+            }
+            if (!bad && chunk > 0) {
+                const unsigned long long incl = (2ull << 62) | (base + tot);
+                asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w + chunk), "l"(incl)
+                             : "memory");
+            }
+            s_base = base;
+            s_bad = bad;
+        }
+        __syncthreads();
+        if (s_bad) {
+            if (tid == 0) {
+                atomicExch(&P.st->abort, 1u);
+                set_status(P.hdr, UNIGS_ERR_TIMEOUT);
+            }
+            break;
+        }
+        const unsigned long long end = s_base + tot;
+        const bool fits = end <= (unsigned long long)P.capacity;
+        if (tid == 0 && (chunk + 1) * 256 >= n_kept) {
+            P.hdr->need = end;
+            P.hdr->n_instances = fits ? (uint32_t)end : 0u;
+            if (!fits) set_status(P.hdr, UNIGS_ERR_CAPACITY);
+        }
+        if (!fits) continue;  // uniform; s_base is not rewritten before the next barrier
+        for (unsigned long long b = (s_base + P.items - 1) / P.items; b * P.items < end; ++b)
+            for (int j = tid; j < bins; j += 256) P.words[b * bins + j] = 0ull;
+        uint32_t o = (uint32_t)s_base + ex;
+        int x0 = 0, y0 = 0, bw = 1, nt = 0, tiles_x = 0;
+        uint32_t g = 0, toff = 0;
+        unsigned long long mask = 0;
+        if (cnt) {
+            const int k = (int)(t / (uint32_t)P.n);
+            g = t - (uint32_t)k * (uint32_t)P.n;
+            const DevCam& cam = P.tab->cam[k];
+            const uint2 r = P.rect[t];
+            x0 = r.x & 0xffff;
+            y0 = r.y & 0xffff;
+            bw = (int)(r.x >> 16) - x0;
+            nt = bw * ((int)(r.y >> 16) - y0);
+            toff = (uint32_t)cam.tile_off;
+            tiles_x = cam.tiles_x;
+            if (nt <= MASK_TILES) mask = P.masks[t];
+        }
+        // slot q of the warp: the pair whose first slot is the last at or before q
+        const uint32_t sc = nt <= MASK_TILES ? cnt : 0u;
+        uint32_t incl = sc;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, s);
+            if (lane >= s) incl += y;
+        }
+        const uint32_t pre = incl - sc;
+        const uint32_t slots = __shfl_sync(0xffffffffu, incl, 31);
+        const uint32_t tile0 = toff + (uint32_t)(y0 * tiles_x + x0);
+        for (uint32_t q0 = 0; q0 < slots; q0 += 32) {
+            const uint32_t q = q0 + lane;
+            int src = 0;
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1) {
+                const uint32_t pc = __shfl_sync(0xffffffffu, pre, src + s);
+                if (pc <= q) src += s;
+            }
+            const uint32_t r = q - __shfl_sync(0xffffffffu, pre, src);
+            const uint32_t so = __shfl_sync(0xffffffffu, o, src);
+            const uint32_t st0 = __shfl_sync(0xffffffffu, tile0, src);
+            const uint32_t sg = __shfl_sync(0xffffffffu, g, src);
+            const int sbw = __shfl_sync(0xffffffffu, bw, src);
+            const int stx = __shfl_sync(0xffffffffu, tiles_x, src);
+            const unsigned long long sm = __shfl_sync(0xffffffffu, mask, src);
+            if (q < slots) {
+                const int j = nth_bit(sm, (int)r);
+                const int ry = j / sbw;
+                put_instance(P, hist, so + r, st0 + (uint32_t)(ry * stx + (j - ry * sbw)), sg);
+            }
+        }
+        const bool large = nt > MASK_TILES && cnt > 0;
+        const unsigned bm = __ballot_sync(0xffffffffu, large);
+        if (bm) {
+            uint32_t slot = 0;
+            if (lane == 0) slot = atomicAdd(&P.st->n_big, (uint32_t)__popc(bm));
+            slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(bm & ((1u << lane) - 1u));
+            if (large) P.big[slot] = make_uint4(t, o, cnt, 0u);
+        }
+        __syncthreads();
+    }
+    flush_hist(P, hist);
+}
+
+// The rectangles of more than MASK_TILES tiles, BIG_SEG tiles per task: a
+// warp repeats the tile test, 32 tiles per step, and takes the positions of
+// the kept ones from the pair's own counter.  (The order of a pair's
+// instances does not reach the sorted lists: each lies in another tile.)
+// Task s * n_big + e is segment s of pair e; a warp's lanes look at every
+// `warps`-th task for those that exist, so that neighbouring tasks (the
+// largest rectangles stand together) go to different warps.
+constexpr int BIG_SEG = 256;
+__global__ void __launch_bounds__(256) emit_big_kernel(const EmitParams P, int max_segs) {
+    __shared__ uint32_t hist[TILE_PASSES_MAX][RS_BINS];
+    const int lane = threadIdx.x & 31;
+    const int64_t n_big = P.st->n_big;
+    if (n_big == 0) return;
+    for (int j = threadIdx.x; j < P.passes * RS_BINS; j += 256) (&hist[0][0])[j] = 0u;
+    __syncthreads();
+    const int64_t n_tasks = n_big * max_segs;
+    const int64_t warps = (int64_t)gridDim.x * 8;
+    // neighbouring warps in different blocks
+    const int64_t warp = (threadIdx.x >> 5) * (int64_t)gridDim.x + blockIdx.x;
+    for (int64_t q0 = warp; q0 < n_tasks; q0 += warps * 32) {
+        const int64_t q = q0 + lane * warps;
+        uint32_t t = 0, o = 0, cnt = 0, e = 0;
+        int seg = 0, x0 = 0, y0 = 0, bw = 1, nt = 0;
+        if (q < n_tasks) {
+            seg = (int)(q / n_big);
+            e = (uint32_t)(q - seg * n_big);
+            const uint4 b = P.big[e];
+            t = b.x;
+            o = b.y;
+            cnt = b.z;
+            const uint2 r = P.rect[t];
+            x0 = r.x & 0xffff;
+            y0 = r.y & 0xffff;
+            bw = (int)(r.x >> 16) - x0;
+            nt = bw * ((int)(r.y >> 16) - y0);
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, seg * BIG_SEG < nt);
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const uint32_t bt = __shfl_sync(0xffffffffu, t, src);
+            const int k = (int)(bt / (uint32_t)P.n);
+            const uint32_t g = bt - (uint32_t)k * (uint32_t)P.n;
+            const DevCam& cam = P.tab->cam[k];
+            const float4* cs = reinterpret_cast<const float4*>(P.cull + (size_t)bt * CULL_FLOATS);
+            const float4 c0 = cs[0], c1 = cs[1];
+            const float cr[CULL_FLOATS] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+            const CullTest ct = cull_test(cr);
+            const int bx0 = __shfl_sync(0xffffffffu, x0, src);
+            const int by0 = __shfl_sync(0xffffffffu, y0, src);
+            const int bbw = __shfl_sync(0xffffffffu, bw, src);
+            const int j1 = __shfl_sync(0xffffffffu, seg, src) * BIG_SEG;
+            const int bn = min(__shfl_sync(0xffffffffu, nt, src), j1 + BIG_SEG);
+            const uint32_t bo = __shfl_sync(0xffffffffu, o, src);
+            const uint32_t bc = __shfl_sync(0xffffffffu, cnt, src);
+            uint32_t* cursor = &P.big[__shfl_sync(0xffffffffu, e, src)].w;
+            for (int j0 = j1; j0 < bn; j0 += 32) {
+                const int j = j0 + lane;
+                const int ry = j / bbw;
+                const int tx = bx0 + (j - ry * bbw), ty = by0 + ry;
+                const bool keep = j < bn && tile_keep(ct, tx, ty, P.tw, P.th);
+                const unsigned m = __ballot_sync(0xffffffffu, keep);
+                if (!m) continue;
+                uint32_t pos = 0;
+                if (lane == 0) pos = atomicAdd(cursor, (uint32_t)__popc(m));
+                pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m & ((1u << lane) - 1u));
+                if (keep && pos < bc)
+                    put_instance(P, hist, bo + pos,
+                                 (uint32_t)cam.tile_off + (uint32_t)(ty * cam.tiles_x + tx), g);
+            }
+        }
+    }
+    flush_hist(P, hist);
+}
+
 // ------------------------------------------------------------ radix sort
+// (the 64-bit pair sort)
 __device__ __forceinline__ uint32_t n_valid(const WsHeader* hdr) {
     return hdr->status == UNIGS_ERR_CAPACITY ? 0u : hdr->n_instances;
 }
@@ -324,16 +769,32 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// Per-tile [start, end) by boundary detection on the sorted keys.
+// Per-tile [start, end) by boundary detection on the sorted tile ids.
 __global__ void __launch_bounds__(256)
-    ranges_kernel(const unsigned long long* __restrict__ keys, const WsHeader* __restrict__ hdr,
-                  uint2* __restrict__ ranges) {
-    const uint32_t n = n_valid(hdr);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t t = (uint32_t)(keys[i] >> 32);
-        if (i == 0 || (uint32_t)(keys[i - 1] >> 32) != t) ranges[t].x = (uint32_t)i;
-        if (i == n - 1 || (uint32_t)(keys[i + 1] >> 32) != t) ranges[t].y = (uint32_t)(i + 1);
+    ranges_kernel(const uint32_t* __restrict__ keys, const WsHeader* __restrict__ hdr,
+                  const SortState* __restrict__ st, uint2* __restrict__ ranges) {
+    const uint32_t n = st->abort ? 0u : hdr->n_instances;
+    // four tile ids per thread (the region is aligned to 256 bytes), and the
+    // one before them
+    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; i < n;
+         i += (int64_t)gridDim.x * blockDim.x * 4) {
+        uint32_t t[5];
+        t[0] = i ? keys[i - 1] : 0xffffffffu;
+        if (i + 4 <= n) {
+            const uint4 q = *reinterpret_cast<const uint4*>(keys + i);
+            t[1] = q.x; t[2] = q.y; t[3] = q.z; t[4] = q.w;
+        } else {
+            for (int j = 0; j < 4; ++j) t[j + 1] = i + j < n ? keys[i + j] : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (i + j >= n) break;
+            if (i + j == 0 || t[j] != t[j + 1]) {
+                ranges[t[j + 1]].x = (uint32_t)(i + j);
+                if (i + j) ranges[t[j]].y = (uint32_t)(i + j);
+            }
+            if (i + j == n - 1) ranges[t[j + 1]].y = n;
+        }
     }
 }
 
@@ -374,53 +835,148 @@ int radix_pass(const unsigned long long* kin, const uint32_t* vin, unsigned long
     return launches + 1;
 }
 
+template <int PER, bool FROM_PAIRS, bool KEYS>
+static void launch_onesweep(const OnesweepParams& P, int64_t n_max, cudaStream_t st) {
+    constexpr int ITEMS = RS_THREADS * PER;
+    const int smem = (int)sizeof(OnesweepSmem<PER>);
+    ensure_smem_limit(reinterpret_cast<const void*>(&onesweep_kernel<PER, FROM_PAIRS, KEYS>), smem);
+    const int64_t chunks = (n_max + ITEMS - 1) / ITEMS, cap = (int64_t)sm_count() * 2;
+    onesweep_kernel<PER, FROM_PAIRS, KEYS>
+        <<<(unsigned)(chunks < cap ? chunks : cap), RS_THREADS, smem, st>>>(P);
+}
+
+template <bool FROM_PAIRS, bool KEYS>
+static void launch_onesweep_n(const OnesweepParams& P, int64_t n_max, cudaStream_t st) {
+    if (rs_per(n_max) == RS_PER_LARGE)
+        launch_onesweep<RS_PER_LARGE, FROM_PAIRS, KEYS>(P, n_max, st);
+    else
+        launch_onesweep<RS_PER_SMALL, FROM_PAIRS, KEYS>(P, n_max, st);
+}
+
 int launch_bin_sort(const unigs_plan& p, void* ws, cudaStream_t st) {
     const int64_t total = p.n * (int64_t)p.n_cams;
     WsHeader* hdr = ws_ptr<WsHeader>(ws, p, OFF_HDR);
     uint2* ranges = ws_ptr<uint2>(ws, p, OFF_RANGES);
-    int launches = 0;
-    cudaMemsetAsync(ranges, 0, sizeof(uint2) * (size_t)p.n_tiles, st);
     if (total == 0 || p.capacity == 0) {
         // no instances: every tile is empty, the schedule is still needed
+        cudaMemsetAsync(ranges, 0, sizeof(uint2) * (size_t)p.n_tiles, st);
         tile_order_kernel<<<1, 1024, 0, st>>>(ranges, p.n_tiles, ws_ptr<uint32_t>(ws, p, OFF_ORDER));
-        return launches + 1;
+        return 1;
     }
-    uint32_t* touched = ws_ptr<uint32_t>(ws, p, OFF_TOUCH);
-    uint32_t* offs = ws_ptr<uint32_t>(ws, p, OFF_OFFS);
-    uint32_t* scan_tmp = ws_ptr<uint32_t>(ws, p, OFF_SCAN);
-    launches += scan_u32(touched, total, scan_tmp, offs, nullptr, st);
-    unsigned long long* keys[2] = {ws_ptr<unsigned long long>(ws, p, OFF_KEYS0),
-                                   ws_ptr<unsigned long long>(ws, p, OFF_KEYS1)};
+    int launches = 0;
+    const uint32_t* touched = ws_ptr<uint32_t>(ws, p, OFF_TOUCH);
+    const uint32_t* zbits = ws_ptr<uint32_t>(ws, p, OFF_ZBITS);
+    SortState* ss = ws_ptr<SortState>(ws, p, OFF_SCAN);
+    unsigned long long* words = ws_ptr<unsigned long long>(ws, p, OFF_HIST);
+    // The depth sort's buffers, dead once the instances are emitted, lie in
+    // the gradient-record region, which only the backward uses.
+    const int64_t pad = (total + 3) / 4 * 4;
+    uint32_t* dz[2] = {ws_ptr<uint32_t>(ws, p, OFF_GREC), ws_ptr<uint32_t>(ws, p, OFF_GREC) + 2 * pad};
+    uint32_t* dt[2] = {dz[0] + pad, dz[1] + pad};
+    unsigned long long* emit_words = reinterpret_cast<unsigned long long*>(dz[0] + 4 * pad);
+    cudaMemsetAsync(ss, 0, sizeof(SortState), st);
+    {
+        const int64_t items = (int64_t)RS_THREADS * rs_per(total);
+        // 16 pairs per thread: each block adds up to 1024 counts to the same
+        // words at its end
+        const int64_t blocks = (total + 8191) / 8192, cap = (int64_t)sm_count() * 4;
+        depth_hist_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 512, 0, st>>>(
+            touched, zbits, total, ss, words, (total + items - 1) / items * 256, emit_words,
+            (total + 255) / 256, ranges, p.n_tiles);
+        ++launches;
+    }
+    OnesweepParams P = {};
+    P.words = words;
+    P.st = ss;
+    P.hdr = hdr;
+    for (int pass = 0; pass < 4; ++pass) {
+        const int src = (pass & 1) ^ 1, dst = src ^ 1;
+        P.kin = pass ? dz[src] : zbits;
+        P.vin = pass ? dt[src] : touched;
+        P.kout = dz[dst];
+        P.vout = dt[dst];
+        P.hist = ss->dhist[pass];
+        P.ticket = &ss->ticket[pass];
+        P.n_ptr = &ss->n_kept;
+        P.n_host = total;
+        P.shift = 8 * pass;
+        P.bits = 8;
+        P.epoch = 1u + pass;
+        if (pass == 0)
+            launch_onesweep_n<true, true>(P, total, st);
+        else if (pass < 3)
+            launch_onesweep_n<false, true>(P, total, st);
+        else
+            launch_onesweep_n<false, false>(P, total, st);
+        ++launches;
+    }
+    int tile_bits = 0;
+    while (((int64_t)1 << tile_bits) < p.n_tiles) ++tile_bits;
+    const int tpasses = (tile_bits + 8) / 9;
+    const int tb = tpasses ? (tile_bits + tpasses - 1) / tpasses : 0;
+    uint32_t* keys[2] = {ws_ptr<uint32_t>(ws, p, OFF_KEYS0), ws_ptr<uint32_t>(ws, p, OFF_KEYS1)};
     uint32_t* vals[2] = {ws_ptr<uint32_t>(ws, p, OFF_VALS0), ws_ptr<uint32_t>(ws, p, OFF_VALS1)};
+    // the last tile pass writes buffer 0
+    int cur = tpasses & 1;
     {
-        const int64_t blocks = (total + 255) / 256;
-        const int grid = (int)(blocks < 152 * 32 ? blocks : 152 * 32);
-        emit_kernel<<<grid, 256, 0, st>>>(ws_ptr<CamTable>(ws, p, OFF_CAM), p.n, p.n_cams,
-                                          p.cfg.tile_w, p.cfg.tile_h, p.capacity, ws_ptr<uint2>(ws, p, OFF_RECT), touched,
-                                          offs, ws_ptr<uint32_t>(ws, p, OFF_ZBITS),
-                                          ws_ptr<float>(ws, p, OFF_CULL), hdr, keys[0], vals[0]);
-        ++launches;
+        EmitParams E;
+        E.tab = ws_ptr<CamTable>(ws, p, OFF_CAM);
+        E.n = p.n;
+        E.tw = p.cfg.tile_w;
+        E.th = p.cfg.tile_h;
+        E.capacity = p.capacity;
+        E.rect = ws_ptr<uint2>(ws, p, OFF_RECT);
+        E.touched = touched;
+        E.masks = cull_masks(ws, p);
+        E.cull = cull_records(ws, p);
+        E.order = dt[1];
+        E.st = ss;
+        E.hdr = hdr;
+        E.emit_words = emit_words;
+        E.big = reinterpret_cast<uint4*>(emit_words + (total + 511) / 512 * 2);
+        E.words = words;
+        E.keys = keys[cur];
+        E.vals = vals[cur];
+        E.passes = tpasses;
+        E.bits = tb;
+        E.items = RS_THREADS * rs_per(p.capacity);
+        const int64_t blocks = (total + 255) / 256, cap = (int64_t)sm_count() * 8;
+        emit_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, st>>>(E);
+        int max_tiles = 0;
+        for (int k = 0; k < p.n_cams; ++k) {
+            const int nt = p.tile_offset[k + 1] - p.tile_offset[k];
+            max_tiles = nt > max_tiles ? nt : max_tiles;
+        }
+        launches += 1;
+        if (max_tiles > MASK_TILES) {
+            emit_big_kernel<<<(unsigned)(blocks * 8 < cap ? blocks * 8 : cap), 256, 0, st>>>(
+                E, (max_tiles + BIG_SEG - 1) / BIG_SEG);
+            ++launches;
+        }
     }
-    const int nb = (int)((p.capacity + SORT_ITEMS - 1) / SORT_ITEMS);
-    uint32_t* hist = ws_ptr<uint32_t>(ws, p, OFF_HIST);
-    for (int pass = 0; pass < p.sort_passes; ++pass) {
-        const int src = pass & 1, dst = src ^ 1;
-        radix_hist_kernel<<<nb, 256, 0, st>>>(keys[src], hdr, 8 * pass, 255u, nb, hist);
-        launches += 1 + scan_u32(hist, (int64_t)nb * 256, scan_tmp, hist, nullptr, st);
-        radix_scatter_kernel<<<nb, 256, 0, st>>>(keys[src], vals[src], keys[dst], vals[dst], hist,
-                                                 hdr, 8 * pass, 255u, nb);
+    for (int pass = 0; pass < tpasses; ++pass) {
+        P.kin = keys[cur];
+        P.vin = vals[cur];
+        P.kout = keys[cur ^ 1];
+        P.vout = vals[cur ^ 1];
+        P.hist = ss->thist[pass];
+        P.ticket = &ss->ticket[TICKET_EMIT + 1 + pass];
+        P.n_ptr = &hdr->n_instances;
+        P.shift = tb * pass;
+        P.bits = tb;
+        P.epoch = 5u + pass;
+        launch_onesweep_n<false, true>(P, p.capacity, st);
         ++launches;
+        cur ^= 1;
     }
-    const int fin = sorted_buffer(p);
     {
-        const int64_t blocks = (p.capacity + 255) / 256;
-        const int grid = (int)(blocks < 152 * 32 ? blocks : 152 * 32);
-        ranges_kernel<<<grid, 256, 0, st>>>(keys[fin], hdr, ranges);
+        const int64_t blocks = (p.capacity + 1023) / 1024;
+        const int grid = (int)(blocks < 152 * 16 ? blocks : 152 * 16);
+        ranges_kernel<<<grid, 256, 0, st>>>(keys[0], hdr, ss, ranges);
         ++launches;
     }
     tile_order_kernel<<<1, 1024, 0, st>>>(ranges, p.n_tiles, ws_ptr<uint32_t>(ws, p, OFF_ORDER));
-    ++launches;
-    return launches;
+    return launches + 1;
 }
 
 }  // namespace unigs

@@ -206,9 +206,12 @@ unigs_status unigs_plan_init(unigs_plan* plan, const unigs_gaussians* g, const u
     while (((int64_t)1 << tile_bits) < tiles) ++tile_bits;
     plan->sort_passes = (32 + tile_bits + 7) / 8;
 
-    const int64_t nb_sort = (cap + SORT_ITEMS - 1) / SORT_ITEMS;
-    const int64_t nb_scan_t = (total + SCAN_ITEMS - 1) / SCAN_ITEMS;
-    const int64_t nb_scan_h = (256 * nb_sort + SCAN_ITEMS - 1) / SCAN_ITEMS;
+    // look-back words of the radix passes: 256 a chunk of pairs, 512 a chunk of
+    // instances
+    const int64_t items_d = (int64_t)RS_THREADS * rs_per(total);
+    const int64_t items_t = (int64_t)RS_THREADS * rs_per(cap);
+    const int64_t words_d = (total + items_d - 1) / items_d * 256;
+    const int64_t words_t = (cap + items_t - 1) / items_t * RS_BINS;
     size_t sizes[OFF_END];
     sizes[OFF_HDR] = sizeof(WsHeader);
     sizes[OFF_CAM] = sizeof(CamTable);
@@ -217,15 +220,17 @@ unigs_status unigs_plan_init(unigs_plan* plan, const unigs_gaussians* g, const u
     sizes[OFF_TOUCH] = sizeof(uint32_t) * (size_t)total;
     sizes[OFF_OFFS] = sizeof(uint32_t) * (size_t)total;
     sizes[OFF_ZBITS] = sizeof(uint32_t) * (size_t)total;
-    sizes[OFF_SCAN] = sizeof(uint32_t) * (size_t)(nb_scan_t > nb_scan_h ? nb_scan_t : nb_scan_h) + 64;
-    sizes[OFF_KEYS0] = sizeof(unsigned long long) * (size_t)cap;
-    sizes[OFF_KEYS1] = sizeof(unsigned long long) * (size_t)cap;
+    sizes[OFF_SCAN] = sizeof(SortState);
+    sizes[OFF_KEYS0] = sizeof(uint32_t) * (size_t)cap;
+    sizes[OFF_KEYS1] = sizeof(uint32_t) * (size_t)cap;
     sizes[OFF_VALS0] = sizeof(uint32_t) * (size_t)cap;
     sizes[OFF_VALS1] = sizeof(uint32_t) * (size_t)cap;
-    sizes[OFF_HIST] = sizeof(uint32_t) * 256 * (size_t)nb_sort;
+    sizes[OFF_HIST] = sizeof(unsigned long long) * (size_t)(words_d > words_t ? words_d : words_t);
     sizes[OFF_RANGES] = sizeof(uint2) * (size_t)tiles;
+    // (the binning's depth sort borrows up to 112 bytes a pair of it)
     sizes[OFF_GREC] = sizeof(double) * GREC_FLOATS * (size_t)total;
-    sizes[OFF_CULL] = sizeof(float) * CULL_FLOATS * (size_t)total;
+    sizes[OFF_CULL] = sizeof(float) * CULL_FLOATS * (size_t)total +
+                      sizeof(unsigned long long) * (size_t)(total + 1);
     // float32 copy of bfloat16 semantic rows, refreshed by every preprocess
     // when an FP32-pipe composite will read it
     sizes[OFF_SEM32] = sem32_needed(*plan) ? sizeof(float) * (size_t)g->n * g->n_sem : 0;
@@ -352,8 +357,13 @@ unigs_status unigs_stats_poll(const unigs_plan* plan, const void* ws, int64_t* p
 
 int32_t unigs_launches_per_step(const unigs_plan* plan) {
     if (!plan) return 0;
-    const int per_pass = 1 + 3 + 1;
-    const int bin = 3 + 1 + per_pass * plan->sort_passes + 1 + 1 /*tile order*/;
+    int tile_bits = 0;
+    while (((int64_t)1 << tile_bits) < plan->n_tiles) ++tile_bits;
+    int emits = 1;
+    for (int k = 0; k < plan->n_cams; ++k)
+        if (plan->tile_offset[k + 1] - plan->tile_offset[k] > MASK_TILES) emits = 2;
+    const int bin = 1 /*depth digits*/ + 4 /*depth passes*/ + emits +
+                    (tile_bits + 8) / 9 /*tile passes*/ + 1 /*ranges*/ + 1 /*tile order*/;
     int conv = 0;
     if (sem32_needed(*plan)) {
         const int64_t cnt = plan->n * (int64_t)plan->n_sem;

@@ -34,7 +34,7 @@ int launch_render_bwd(const unigs_plan& p, const unigs_gaussians& g, void* ws,
                       const unigs_outputs& fwd, const unigs_grad_outputs& go,
                       const unigs_param_grads& grads, cudaStream_t st);
 
-// One stable LSD radix pass over the n = hdr->n_instances pairs (n read on
+// One stable LSD radix pass of the 64-bit pair sort over the n = hdr->n_instances pairs (n read on
 // the device; 0 when hdr->status reports a capacity overflow) on the digit
 // (key >> shift) & dmask (dmask 255 for a whole byte, 2^b - 1 to sort by b < 8
 // bits): per-block digit histograms, their exclusive scan, stable scatter.  nb
@@ -69,8 +69,5 @@ int sm_count();
 // current device, once per (kernel, device); thread-safe.  Returns the CUDA
 // error of the attribute call (cudaSuccess when it was already set).
 cudaError_t ensure_smem_limit(const void* func, int bytes);
-
-// Index of the buffer (0/1) that holds the sorted keys/values after the sort.
-inline int sorted_buffer(const unigs_plan& p) { return p.sort_passes & 1; }
 
 }  // namespace unigs

@@ -803,8 +803,7 @@ int launch_render_bwd(const unigs_plan& p, const unigs_gaussians& g, void* ws,
         P.rec = ws_ptr<float>(ws, p, OFF_REC);
         // bfloat16 logits are read from their float32 copy (made by the preprocess)
         P.sem = p.feat_dtype ? ws_ptr<float>(ws, p, OFF_SEM32) : static_cast<const float*>(g.sem);
-        P.vals = sorted_buffer(p) ? ws_ptr<uint32_t>(ws, p, OFF_VALS1)
-                                  : ws_ptr<uint32_t>(ws, p, OFF_VALS0);
+        P.vals = ws_ptr<uint32_t>(ws, p, OFF_VALS0);
         P.ranges = ws_ptr<uint2>(ws, p, OFF_RANGES);
         P.order = ws_ptr<uint32_t>(ws, p, OFF_ORDER);
         WsHeader* hdr = ws_ptr<WsHeader>(ws, p, OFF_HDR);

@@ -460,7 +460,7 @@ int launch_render_fwd_tc(const unigs_plan& p, const unigs_gaussians& g, void* ws
     P.n_tiles = p.n_tiles;
     P.rec = ws_ptr<float>(ws, p, OFF_REC);
     P.sem = g.sem;
-    P.vals = sorted_buffer(p) ? ws_ptr<uint32_t>(ws, p, OFF_VALS1) : ws_ptr<uint32_t>(ws, p, OFF_VALS0);
+    P.vals = ws_ptr<uint32_t>(ws, p, OFF_VALS0);
     P.ranges = ws_ptr<uint2>(ws, p, OFF_RANGES);
     P.order = ws_ptr<uint32_t>(ws, p, OFF_ORDER);
     WsHeader* hdr = ws_ptr<WsHeader>(ws, p, OFF_HDR);

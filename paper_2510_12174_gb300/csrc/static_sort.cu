@@ -1,5 +1,5 @@
-// unigs_sort_pairs_static: the library's stable radix sort of (key, value)
-// pairs, with its scratch memory in a file-scope device array instead of a
+// unigs_sort_pairs_static: a stable radix sort of 64-bit (key, value) pairs
+// with its scratch memory in a file-scope device array instead of a
 // caller-allocated workspace.
 //
 // It exists for callers that cannot allocate device memory at the point of

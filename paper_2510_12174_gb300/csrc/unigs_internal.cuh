@@ -184,55 +184,102 @@ __device__ __forceinline__ float cull_q(float kA, float kB, float kC, float dx, 
                      __fmul_rn(__fmul_rn(kC, dy), dy));
 }
 
-__device__ __forceinline__ bool tile_keep(const float* __restrict__ cr, int tx, int ty, int tw,
-                                          int th) {
-    if (cr[C_NOCULL] != 0.f) return true;
-    const float mx = cr[C_MX], my = cr[C_MY], kA = cr[C_KA], kB = cr[C_KB], kC = cr[C_KC];
-    const float X0 = (float)(tx * tw), X1 = (float)(tx * tw + tw - 1);
-    const float Y0 = (float)(ty * th), Y1 = (float)(ty * th + th - 1);
-    float qmin;
-    if (X0 <= mx && mx <= X1 && Y0 <= my && my <= Y1) {
-        qmin = 0.f;
-    } else {
-        const float ylo = __fsub_rn(Y0, my), yhi = __fsub_rn(Y1, my);
-        const float xlo = __fsub_rn(X0, mx), xhi = __fsub_rn(X1, mx);
-        float q[4];
-        {
-            const float dx = xlo;
-            const float dy = fminf(fmaxf(__fdiv_rn(-__fmul_rn(kB, dx), kC), ylo), yhi);
-            q[0] = cull_q(kA, kB, kC, dx, dy);
-        }
-        {
-            const float dx = xhi;
-            const float dy = fminf(fmaxf(__fdiv_rn(-__fmul_rn(kB, dx), kC), ylo), yhi);
-            q[1] = cull_q(kA, kB, kC, dx, dy);
-        }
-        {
-            const float dy = ylo;
-            const float dx = fminf(fmaxf(__fdiv_rn(-__fmul_rn(kB, dy), kA), xlo), xhi);
-            q[2] = cull_q(kA, kB, kC, dx, dy);
-        }
-        {
-            const float dy = yhi;
-            const float dx = fminf(fmaxf(__fdiv_rn(-__fmul_rn(kB, dy), kA), xlo), xhi);
-            q[3] = cull_q(kA, kB, kC, dx, dy);
-        }
-        qmin = fminf(fminf(q[0], q[1]), fminf(q[2], q[3]));
+// The record's conic with correctly rounded reciprocals of its diagonal
+// (0 where a reciprocal or a quotient by it could leave the normal range).
+struct CullTest {
+    float mx, my, kA, kB, kC, qlim, yA, yC;
+    bool nocull;
+};
+__device__ __forceinline__ CullTest cull_test(const float* __restrict__ cr) {
+    CullTest c = {cr[C_MX], cr[C_MY], cr[C_KA], cr[C_KB], cr[C_KC], cr[C_QLIM], 0.f, 0.f,
+                  cr[C_NOCULL] != 0.f};
+    constexpr float LO = 0x1p-60f, HI = 0x1p60f;
+    if (c.kA >= LO && c.kA <= HI && c.kC >= LO && c.kC <= HI) {
+        c.yA = __frcp_rn(c.kA);
+        c.yC = __frcp_rn(c.kC);
     }
-    return qmin <= cr[C_QLIM];
+    return c;
 }
 
-constexpr int SORT_ITEMS = 2048;   // keys per sort block (256 threads x 8)
-// Tile rectangles with more tiles than this are culled-tested and emitted by
-// the whole warp (32 tiles per step) rather than by their own thread: a lane
-// with a long serial loop would hold its warp (measured: 4 beats 8, 16, 32).
-constexpr int COOP_TILES = 4;
+// n / d rounded, y the correctly rounded 1 / d: the quotient n y corrected by
+// its exact residual is the rounded quotient (Markstein 1990).  (For |n| below
+// 2^-100 the residual may be inexact; such a step moves q by nothing.)  Three
+// instructions, where the general division takes about twelve.
+__device__ __forceinline__ float div_recip(float n, float d, float y) {
+    const float q = __fmul_rn(n, y);
+    return __fmaf_rn(__fmaf_rn(-d, q, n), y, q);
+}
+
+__device__ __forceinline__ bool tile_keep(const CullTest& c, int tx, int ty, int tw, int th) {
+    if (c.nocull) return true;
+    const float X0 = (float)(tx * tw), X1 = (float)(tx * tw + tw - 1);
+    const float Y0 = (float)(ty * th), Y1 = (float)(ty * th + th - 1);
+    if (X0 <= c.mx && c.mx <= X1 && Y0 <= c.my && c.my <= Y1) return 0.f <= c.qlim;
+    const float ylo = __fsub_rn(Y0, c.my), yhi = __fsub_rn(Y1, c.my);
+    const float xlo = __fsub_rn(X0, c.mx), xhi = __fsub_rn(X1, c.mx);
+    const bool fast = c.yA != 0.f;
+    float q[4];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const float dx = e ? xhi : xlo;
+        const float n = -__fmul_rn(c.kB, dx);
+        const float d = fast ? div_recip(n, c.kC, c.yC) : __fdiv_rn(n, c.kC);
+        q[e] = cull_q(c.kA, c.kB, c.kC, dx, fminf(fmaxf(d, ylo), yhi));
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const float dy = e ? yhi : ylo;
+        const float n = -__fmul_rn(c.kB, dy);
+        const float d = fast ? div_recip(n, c.kA, c.yA) : __fdiv_rn(n, c.kA);
+        q[2 + e] = cull_q(c.kA, c.kB, c.kC, fminf(fmaxf(d, xlo), xhi), dy);
+    }
+    return fminf(fminf(q[0], q[1]), fminf(q[2], q[3])) <= c.qlim;
+}
+
 constexpr int SCAN_ITEMS = 4096;   // elements per scan block (256 threads x 16)
 constexpr int LOSS_MAX_BLOCKS = 2048;  // block partials of the loss reduction
+// Rectangles of at most this many tiles carry a bit mask of their kept tiles
+// from the preprocess to the emission, which then repeats no tile test; larger
+// ones (rare) carry the test's record.
+constexpr int MASK_TILES = 64;
+constexpr int SORT_ITEMS = 2048;   // keys per block of the 64-bit pair sort (256 threads x 8)
+// Blocks of the single-kernel radix passes: RS_THREADS threads (one per digit
+// value at most) of RS_PER keys.
+constexpr int RS_THREADS = 512;
+constexpr int RS_WARPS = RS_THREADS / 32;
+constexpr int RS_BINS = 512;
+constexpr int RS_PER_LARGE = 16, RS_PER_SMALL = 4;
+// Keys per thread for an array of at most n keys: below about two full waves
+// of large blocks (2 blocks of 8192 keys on each of 152 SMs) small blocks
+// spread the keys over more SMs.
+__host__ __device__ constexpr int rs_per(int64_t n) {
+    return n >= 4 * 1000 * 1000 ? RS_PER_LARGE : RS_PER_SMALL;
+}
+constexpr int TILE_PASSES_MAX = 4;  // ceil(31 tile bits / 9)
+constexpr int TICKET_EMIT = 4;      // tickets 0..3: depth passes, then emission, tile passes
 
+// State of one binning, zeroed at its start.
+struct SortState {
+    uint32_t ticket[TICKET_EMIT + 1 + TILE_PASSES_MAX + 3];
+    uint32_t n_kept;                 // pairs with a kept tile
+    uint32_t n_big;                  // kept pairs of more than MASK_TILES tiles
+    uint32_t abort;                  // a bounded wait gave up
+    uint32_t pad;
+    uint32_t dhist[4][256];          // depth digits of the kept pairs
+    uint32_t thist[TILE_PASSES_MAX][RS_BINS];  // tile digits of the instances
+};
 template <typename T>
 __host__ __device__ inline T* ws_ptr(void* ws, const unigs_plan& p, int region) {
     return reinterpret_cast<T*>(static_cast<char*>(ws) + p.off[region]);
+}
+
+// The tile-test region: a kept-tile mask per pair, then a test record per pair.
+__host__ inline unsigned long long* cull_masks(void* ws, const unigs_plan& p) {
+    return ws_ptr<unsigned long long>(ws, p, OFF_CULL);
+}
+__host__ inline float* cull_records(void* ws, const unigs_plan& p) {
+    const size_t total = (size_t)p.n * (size_t)p.n_cams;
+    return reinterpret_cast<float*>(cull_masks(ws, p) + (total + 1) / 2 * 2);
 }
 
 __device__ inline const DevCam& cam_of_tile(const CamTable* tab, int n_cams, int64_t gtile,

@@ -279,14 +279,21 @@ class Renderer:
         s, _ = self.status()
         abi.check(s, "status")
         n = int(self.ws[self.plan.off[0] + 4: self.plan.off[0] + 8].view(torch.int32).item())
-        fin = int(self.plan.sort_passes) & 1
-        ko = self.plan.off[8 + fin]
-        vo = self.plan.off[10 + fin]
-        keys = self.ws[ko: ko + 8 * n].view(torch.int64).cpu().numpy().view(np.uint64)
-        vals = self.ws[vo: vo + 4 * n].view(torch.int32).cpu().numpy().view(np.uint32)
-        ro = self.plan.off[13]
+
+        def words(region, count):
+            o = self.plan.off[region]
+            return self.ws[o: o + 4 * count].view(torch.int32).cpu().numpy().view(np.uint32)
+
+        # the workspace holds the sorted tile ids and Gaussian indices; a key's
+        # depth bits are those of its (camera, Gaussian) pair
+        tiles, vals = words(8, n), words(10, n)
         nt = int(self.plan.n_tiles)
-        ranges = self.ws[ro: ro + 8 * nt].view(torch.int32).cpu().numpy().view(np.uint32)
+        ranges = words(13, 2 * nt)
+        n_cams = len(self.cam_list)
+        offs = np.array([int(self.plan.tile_offset[k]) for k in range(n_cams)])
+        cam = np.searchsorted(offs, tiles, side="right") - 1
+        z = words(6, self.scene.n * n_cams)[cam * self.scene.n + vals]
+        keys = tiles.astype(np.uint64) << np.uint64(32) | z
         return keys, vals, ranges.reshape(nt, 2)
 
 
