@@ -46,23 +46,34 @@ __device__ __forceinline__ void pixel_cam(const LossParams& P, int64_t gp, int* 
 
 __device__ __forceinline__ float sgn(float x) { return (float)((x > 0.f) - (x < 0.f)); }
 
-// The logits of one pixel (planar channels) into registers, padding with
-// -inf, and their maximum and sum of exponentials.
-template <int NS>
+// The logits of one pixel (planar channels) into registers, padded with -inf,
+// and their maximum (four chains, so that it does not serialise 64 steps).
+// FULL: C == NS, no channel is tested.
+template <int NS, bool FULL>
 __device__ __forceinline__ void pixel_logits(const float* O, int64_t hw, int C, float (&o)[NS],
-                                             float* mx_out, float* z_out) {
-    float mx = -INFINITY;
+                                             float* mx_out) {
 #pragma unroll
     for (int c = 0; c < NS; ++c) {
-        o[c] = c < C ? O[(int64_t)c * hw] : -INFINITY;
-        mx = fmaxf(mx, o[c]);
+        o[c] = FULL || c < C ? *O : -INFINITY;
+        O += hw;
     }
+    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int c = 0; c < NS; ++c) mx[c & 3] = fmaxf(mx[c & 3], o[c]);
+    *mx_out = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+}
+
+// o[c] <- exp(o[c] - mx), returning their sum (a padded channel is exp(-inf) = 0).
+template <int NS, bool FULL>
+__device__ __forceinline__ float exp_sum(float (&o)[NS], float mx, int C) {
     float z = 0.f;
 #pragma unroll
     for (int c = 0; c < NS; ++c)
-        if (c < C) z += expf(o[c] - mx);
-    *mx_out = mx;
-    *z_out = z;
+        if (FULL || c < C) {
+            o[c] = expf(o[c] - mx);
+            z += o[c];
+        }
+    return z;
 }
 
 __device__ __forceinline__ float block_sum(float v, float* sh) {
@@ -78,7 +89,13 @@ __device__ __forceinline__ float block_sum(float v, float* sh) {
     return s;  // valid in thread 0
 }
 
-template <int NS>
+// Per 32 pixels of 64 logits the loads and stores take some 60 ns of an SM's
+// share of the memory bandwidth, about as long as 20 instructions per logit
+// take to issue.  So each exponential is formed once, the channel tests are
+// compiled out where C fills the register array, and the label's logit is read
+// again instead of selected.  The pixels of a thread and the order of its sums
+// do not depend on any of this.
+template <int NS, bool FULL>
 __global__ void __launch_bounds__(LOSS_THREADS) loss_sums_kernel(const LossParams P) {
     __shared__ float sh[32];
     float acc[LOSS_SUMS] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -109,13 +126,11 @@ __global__ void __launch_bounds__(LOSS_THREADS) loss_sums_kernel(const LossParam
             const int lab = P.tgt.label[gp];
             if (lab >= 0 && lab < P.n_sem) {
                 constexpr int N1 = NS > 0 ? NS : 1;
-                float o[N1], mx, z;
-                pixel_logits<N1>(P.logits + po * P.n_sem + idx, hw, P.n_sem, o, &mx, &z);
-                float ol = 0.f;
-#pragma unroll
-                for (int c = 0; c < N1; ++c)
-                    if (c == lab) ol = o[c];
-                acc[4] += mx + logf(z) - ol;
+                const float* O = P.logits + po * P.n_sem + idx;
+                float o[N1], mx;
+                pixel_logits<N1, FULL>(O, hw, P.n_sem, o, &mx);
+                const float z = exp_sum<N1, FULL>(o, mx, P.n_sem);
+                acc[4] += mx + logf(z) - O[lab * hw];
                 acc[5] += 1.f;
             }
         }
@@ -169,7 +184,7 @@ __global__ void __launch_bounds__(LOSS_THREADS) loss_finalize_kernel(const LossP
     r[13] = r[14] = r[15] = 0.f;
 }
 
-template <int NS>
+template <int NS, bool FULL>
 __global__ void __launch_bounds__(LOSS_THREADS) loss_grad_kernel(const LossParams P) {
     const float* r = P.record;
     const float Pf = (float)P.n_pixels;
@@ -208,29 +223,39 @@ __global__ void __launch_bounds__(LOSS_THREADS) loss_grad_kernel(const LossParam
             float* G = P.g.logits + po * P.n_sem + idx;
             const int lab = P.tgt.label ? P.tgt.label[gp] : -1;
             if (lab >= 0 && lab < P.n_sem) {
-                float o[N1], mx, z;
-                pixel_logits<N1>(P.logits + po * P.n_sem + idx, hw, P.n_sem, o, &mx, &z);
-                const float iz = a_s / z;
+                float o[N1], mx;
+                pixel_logits<N1, FULL>(P.logits + po * P.n_sem + idx, hw, P.n_sem, o, &mx);
+                const float iz = a_s / exp_sum<N1, FULL>(o, mx, P.n_sem);
 #pragma unroll
-                for (int c = 0; c < N1; ++c)
-                    if (c < P.n_sem) {
-                        const float p = expf(o[c] - mx) * iz;
-                        G[(int64_t)c * hw] = c == lab ? p - a_s : p;
-                    }
+                for (int c = 0; c < N1; ++c) {
+                    const float p = o[c] * iz;
+                    if (FULL || c < P.n_sem) *G = c == lab ? p - a_s : p;
+                    G += hw;
+                }
             } else {
 #pragma unroll
-                for (int c = 0; c < N1; ++c)
-                    if (c < P.n_sem) G[(int64_t)c * hw] = 0.f;
+                for (int c = 0; c < N1; ++c) {
+                    if (FULL || c < P.n_sem) *G = 0.f;
+                    G += hw;
+                }
             }
         }
     }
 }
 
+template <int NS, bool FULL>
+static void launch_loss_f(const LossParams& P, int blocks, cudaStream_t st) {
+    loss_sums_kernel<NS, FULL><<<(unsigned)blocks, LOSS_THREADS, 0, st>>>(P);
+    loss_finalize_kernel<<<1, LOSS_THREADS, 0, st>>>(P, blocks);
+    loss_grad_kernel<NS, FULL><<<(unsigned)blocks, LOSS_THREADS, 0, st>>>(P);
+}
+
 template <int NS>
 static void launch_loss_t(const LossParams& P, int blocks, cudaStream_t st) {
-    loss_sums_kernel<NS><<<(unsigned)blocks, LOSS_THREADS, 0, st>>>(P);
-    loss_finalize_kernel<<<1, LOSS_THREADS, 0, st>>>(P, blocks);
-    loss_grad_kernel<NS><<<(unsigned)blocks, LOSS_THREADS, 0, st>>>(P);
+    if (P.n_sem == NS)
+        launch_loss_f<NS, true>(P, blocks, st);
+    else
+        launch_loss_f<NS, false>(P, blocks, st);
 }
 
 int launch_loss(const unigs_plan& p, const unigs_outputs& out, const float* normal_d,
