@@ -47,13 +47,21 @@ __device__ __forceinline__ float bwd_pair(const float* __restrict__ rc, const Pi
                                           float& T, float& Sacc, float (&gv)[32]) {
     const float om = 1.f - alpha;
     // om >= 1 - alpha_max.  The restoration T <- T / om runs along
-    // the whole list, so it keeps the correctly rounded division
-    // (with an approximate quotient the worst cancelling rotation
+    // the whole list, so it takes the correctly rounded quotient
+    // (with an approximate one the worst cancelling rotation
     // gradient of a 200k-Gaussian test scene drifted 2.5x further
-    // from the float64 reference); dL/dalpha takes an approximate
-    // reciprocal
+    // from the float64 reference); dL/dalpha takes the approximate
+    // reciprocal.  A Newton step rounds the reciprocal correctly but
+    // for cases within 2^-20 of a tie; with the quotient's residual,
+    // exact by the fused multiply-add, the corrected quotient is then
+    // the rounded one (Markstein 1990).  T is in [T_min, 1] and om in
+    // [1 - alpha_max, 1], so the range tests of a general division
+    // have nothing to find.
     const float rom = rcp_ftz(om);
-    if (contrib) T = __fdiv_rn(T, om);
+    const float ryn = __fmaf_rn(__fmaf_rn(-om, rom, 1.f), rom, rom);
+    const float q0 = __fmul_rn(T, ryn);
+    const float Tq = __fmaf_rn(__fmaf_rn(-om, q0, T), ryn, q0);
+    if (contrib) T = Tq;
     const float w = contrib ? alpha * T : 0.f;
     PairGeom G;
     pair_geometry(rc, xt, yt, dx, dy, G);

@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(256, (B <= 8 ? 3 : 2)) render_bwd_kernel(const
         PixelUp up = {{0.f, 0.f, 0.f}, 0.f, {0.f, 0.f, 0.f}, 0.f};
         // upstream logit gradients of this pixel -> shared memory row tid (zero
         // padded), read by this thread for G_i and by the warp's channel gather
-#pragma unroll 8
+#pragma unroll 16
         for (int c = 0; c < NS; ++c)
             S.gO[go_index<NS>(tid, c)] = (inside && P.go.logits && c < P.n_sem)
                                ? P.go.logits[pix * (int64_t)P.n_sem + c * HW + idx] : 0.f;

@@ -35,12 +35,12 @@
 //       (p / 8) * 2048 + chunk * 128 + (p % 8) * 16: K-major for MMA 1
 //       (M = pixels: lbo 128, sbo 2048) and, read transposed, MN-major for
 //       MMA 2 (M = K-entries along a row: sbo 128; K = pixels: lbo 2048);
-//   wb: W^T per split, K-major (N = Gaussians, K = pixels): Gaussian j,
+//   wb: W^T per split, K-major (N = Gaussians, K = pixels; the lo split follows the hi split): Gaussian j,
 //       pixel p at (j / 8) * 4096 + (p / 8) * 128 + (j % 8) * 16 + (p % 8) * 2;
 //   fb: F, K-major (N = Gaussians, K = channels), re-laid from the staged
 //       rows by the staging warp.
 // Tensor memory (float32 accumulators): Gsem for (buffer, M-tile) at column (2 buffer + M-tile) B,
-// dL/dF for buffer at column 4 B + buffer B; pixel thread tid owns lane tid %
+// dL/dF for buffer at column 4 B + 2 B buffer (w_hi, then w_lo); pixel thread tid owns lane tid %
 // 128 of M-tile tid / 128.
 //
 // Warps 0-7 walk the pixels (one pixel per thread, as in the FP32-pipe
@@ -94,6 +94,7 @@ struct BwdTcSmem {
     static constexpr int SBO_G = KCH * 128;      // between 8-pixel groups of ga
     static constexpr int SBO_W = 32 * 128;       // between 8-Gaussian groups of W^T
     static constexpr int W_BYTES = B * 256 * 2;  // one split of W^T
+    static_assert(W_BYTES == (B / 8) * SBO_W, "the splits are consecutive 8-Gaussian groups");
     static constexpr int SBO_F = (NS / 8) * 128; // between 8-Gaussian groups of F
     static_assert(2 * NS <= 8 * KCH, "the upstream rows hold NS hi and NS lo entries");
     __align__(1024) unsigned char ga[32 * SBO_G];
@@ -170,9 +171,9 @@ __global__ void __launch_bounds__(BTC_THREADS, BTC_CTAS_PER_SM)
     render_bwd_tc_kernel(const BwdTcParams P) {
     using Sm = BwdTcSmem<NS>;
     constexpr int B = BTC_BATCH;
-    constexpr uint32_t NCOLS = 128;  // Gsem 4 B + dL/dF 2 B = 96 columns
+    constexpr uint32_t NCOLS = 128;  // Gsem 4 B + dL/dF 2 x 2 B columns
     constexpr uint32_t IDESC1 = idesc_f16_f32(128, B);
-    constexpr uint32_t IDESC2 = idesc_f16_f32(128, B) | IDESC_A_MN;
+    constexpr uint32_t IDESC2 = idesc_f16_f32(128, 2 * B) | IDESC_A_MN;
     constexpr float W_SCALE = 16384.f, W_UNSCALE = 1.f / 16384.f;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Sm& S = *reinterpret_cast<Sm*>(smem_raw);
@@ -245,21 +246,40 @@ __global__ void __launch_bounds__(BTC_THREADS, BTC_CTAS_PER_SM)
         float T = 1.f;
         uint32_t last = 0;
         PixelUp up = {{0.f, 0.f, 0.f}, 0.f, {0.f, 0.f, 0.f}, 0.f};
+        uint32_t wlast = 0;  // the warp's own last list position
         const float* g_log = P.go.logits ? P.go.logits + pix * (int64_t)P.n_sem + idx : nullptr;
+        constexpr int GH = NS <= 16 ? NS : NS / 2;
+        auto load_gl = [&](int c0, float (&gl)[GH]) {
+            const float* src = g_log + c0 * HW;
+#pragma unroll
+            for (int c = 0; c < GH; ++c) {
+                gl[c] = (inside && g_log && c0 + c < P.n_sem) ? *src : 0.f;
+                src += HW;
+            }
+        };
         if (!stager) {
-            // the tile's largest upstream logit gradient (for its scale)
-            float gm = 0.f;
-            if (inside && g_log)
-                for (int c = 0; c < P.n_sem; ++c) gm = fmaxf(gm, fabsf(g_log[c * HW]));
-            if (gm > 0.f) atomicMax(&S.gmax, __float_as_uint(gm));
             if (inside) {
                 T = P.T_final[pix + idx];
                 last = P.n_contrib[pix + idx];
                 load_pixel_up(P.go, pix, HW, idx, up);
             }
-            if (last) atomicMax(&S.max_last, last);
+            // the largest of the tile's upstream logit gradients (for its
+            // scale), up to 32 loads in flight at once
+            float gm = 0.f;
+#pragma unroll 1
+            for (int c0 = 0; c0 < NS; c0 += GH) {
+                float gl[GH];
+                load_gl(c0, gl);
+#pragma unroll
+                for (int c = 0; c < GH; ++c) gm = fmaxf(gm, fabsf(gl[c]));
+            }
+            const uint32_t wgm = __reduce_max_sync(0xffffffffu, __float_as_uint(gm));
+            wlast = __reduce_max_sync(0xffffffffu, last);
+            if (lane == 0) {
+                atomicMax(&S.gmax, wgm);
+                atomicMax(&S.max_last, wlast);
+            }
         }
-        const uint32_t wlast = __reduce_max_sync(0xffffffffu, last);
         __syncthreads();
         const int kg = scale_exp(__uint_as_float(S.gmax));
         const float ginv = pow2f(-kg);
@@ -268,22 +288,21 @@ __global__ void __launch_bounds__(BTC_THREADS, BTC_CTAS_PER_SM)
             // K-entries
             const float sg = pow2f(kg);
             unsigned char* grow = S.ga + (ptid >> 3) * Sm::SBO_G + (ptid & 7) * 16;
+#pragma unroll 1
+            for (int c0 = 0; c0 < NS; c0 += GH) {
+                float gl[GH];
+                load_gl(c0, gl);
 #pragma unroll
-            for (int kc = 0; kc < NS / 8; ++kc) {
-                uint32_t h[4], l[4];
+                for (int q = 0; q < GH / 8; ++q) {
+                    const int kc = c0 / 8 + q;
+                    uint32_t h[4], l[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float f[2];
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const int c = 8 * kc + 2 * e + q;
-                        f[q] = (inside && g_log && c < P.n_sem) ? g_log[c * HW] * sg : 0.f;
-                    }
-                    split_f16x2(f[0], f[1], h[e], l[e]);
+                    for (int e = 0; e < 4; ++e)
+                        split_f16x2(gl[8 * q + 2 * e] * sg, gl[8 * q + 2 * e + 1] * sg, h[e], l[e]);
+                    *reinterpret_cast<uint4*>(grow + kc * 128) = make_uint4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<uint4*>(grow + (NS / 8 + kc) * 128) =
+                        make_uint4(l[0], l[1], l[2], l[3]);
                 }
-                *reinterpret_cast<uint4*>(grow + kc * 128) = make_uint4(h[0], h[1], h[2], h[3]);
-                *reinterpret_cast<uint4*>(grow + (NS / 8 + kc) * 128) =
-                    make_uint4(l[0], l[1], l[2], l[3]);
             }
 #pragma unroll
             for (int kc = NS / 4; kc < Sm::KCH; ++kc)
@@ -307,17 +326,16 @@ __global__ void __launch_bounds__(BTC_THREADS, BTC_CTAS_PER_SM)
                 }
                 if (lane == 0) {
                     tc_fence_after_sync();
-                    const uint32_t d = tmem + 4 * B + (uint32_t)(bf * B);
+                    const uint32_t d = tmem + 4 * B + (uint32_t)(bf * 2 * B);
+                    // the hi and lo parts of W^T as one operand of N = 2 B
+                    // columns, so that the upstream rows are read once
 #pragma unroll 1
                     for (int ks = 0; ks < 16; ++ks) {
                         const uint64_t a = smem_desc_kmajor(S.ga + ks * 2 * Sm::SBO_G,
                                                             Sm::SBO_G, 128);
-#pragma unroll
-                        for (int s = 0; s < 2; ++s) {
-                            const uint64_t w = smem_desc_kmajor(&S.wb[bf][s][0] + ks * 256, 128,
-                                                                Sm::SBO_W);
-                            mma_bf16(d, a, w, IDESC2, (ks > 0 || s > 0) ? 1u : 0u);
-                        }
+                        const uint64_t w = smem_desc_kmajor(&S.wb[bf][0][0] + ks * 256, 128,
+                                                            Sm::SBO_W);
+                        mma_bf16(d, a, w, IDESC2, ks > 0 ? 1u : 0u);
                     }
                     mma_commit(&S.d2_bar[bf]);
                 }
@@ -414,8 +432,11 @@ __global__ void __launch_bounds__(BTC_THREADS, BTC_CTAS_PER_SM)
                     return;
                 }
                 tc_fence_after_sync();
-                float dv[8];
-                tmem_ld8(tmem + lane_addr + 4 * B + (uint32_t)(bf * B + ccol), dv);
+                float dv[8], dl[8];
+                tmem_ld8(tmem + lane_addr + 4 * B + (uint32_t)(bf * 2 * B + ccol), dv);
+                tmem_ld8(tmem + lane_addr + 4 * B + (uint32_t)(bf * 2 * B + B + ccol), dl);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) dv[q] += dl[q];
                 if (crow_ok) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
