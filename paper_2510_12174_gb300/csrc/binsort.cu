@@ -141,6 +141,11 @@ __device__ __forceinline__ unsigned long long lb_load(const unsigned long long* 
     return v;
 }
 
+// A word of the emission's look-back: state << 62 | count.
+__device__ __forceinline__ void emit_store(unsigned long long* w, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"(v) : "memory");
+}
+
 constexpr uint32_t LB_WAIT_LIMIT = 1u << 20;  // polls of one word, about a second
 constexpr int LB_WIDE = 8;                    // predecessors read per step
 
@@ -195,13 +200,24 @@ __global__ void __launch_bounds__(512)
     for (int64_t i = i0; i < n_emit_words; i += stride) emit_words[i] = 0ull;
     for (int64_t i = i0; i < n_tiles; i += stride) ranges[i] = make_uint2(0u, 0u);
     uint32_t kept = 0;
-    for (int64_t i = i0; i < total; i += stride) {
-        if (touched[i] == 0) continue;
-        const uint32_t z = zbits[i];
+    auto count = [&](uint32_t cnt, uint32_t z) {
+        if (cnt == 0) return;
         ++kept;
 #pragma unroll
         for (int p = 0; p < 4; ++p) atomicAdd(&h[p][(z >> (8 * p)) & 255u], 1u);
+    };
+    // four pairs a load (the regions start at multiples of 256 bytes)
+    const int64_t n4 = total / 4;
+#pragma unroll 2
+    for (int64_t i = i0; i < n4; i += stride) {
+        const uint4 c = reinterpret_cast<const uint4*>(touched)[i];
+        const uint4 z = reinterpret_cast<const uint4*>(zbits)[i];
+        count(c.x, z.x);
+        count(c.y, z.y);
+        count(c.z, z.z);
+        count(c.w, z.w);
     }
+    if (i0 < total - 4 * n4) count(touched[4 * n4 + i0], zbits[4 * n4 + i0]);
     kept = __reduce_add_sync(0xffffffffu, kept);
     if ((threadIdx.x & 31) == 0 && kept) atomicAdd(&st->n_kept, kept);
     __syncthreads();
@@ -460,44 +476,47 @@ __global__ void __launch_bounds__(256) emit_kernel(const EmitParams P) {
         const uint32_t ex = block_exclusive_scan(cnt, sw, &tot);
         // the instances of all chunks may exceed 32 bits (then far over the
         // capacity): the words' 62-bit counts are kept apart from the state
-        // in the two top bits
-        if (tid == 0) {
+        // in the two top bits.  The first warp reads 64 predecessors a step
+        if (tid < 32) {
             constexpr unsigned long long VAL = (1ull << 62) - 1ull;
             unsigned long long base = 0;
             unsigned long long* w = P.emit_words;
-            int bad = 0;
-            const unsigned long long own = ((chunk == 0 ? 2ull : 1ull) << 62) | tot;
-            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w + chunk), "l"(own) : "memory");
+            bool bad = false;
+            if (lane == 0) emit_store(w + chunk, (chunk == 0 ? 2ull : 1ull) << 62 | tot);
             uint32_t polls = 0;
             for (int64_t p = chunk - 1; p >= 0;) {
-                unsigned long long v[LB_WIDE];
+                // lane l: predecessors p - 2 l and p - 2 l - 1
+                const int64_t p0 = p - 2 * lane;
+                const unsigned long long v0 = p0 >= 0 ? lb_load(w + p0) : 2ull << 62;
+                const unsigned long long v1 = p0 >= 1 ? lb_load(w + p0 - 1) : 2ull << 62;
+                const int s0 = (int)(v0 >> 62), s1 = (int)(v1 >> 62);
+                // the lanes up to the first inclusive prefix or unwritten word
+                const bool stop0 = s0 != 1, stop1 = s1 != 1;
+                const uint32_t stops = __ballot_sync(0xffffffffu, stop0 || stop1);
+                const int at = stops ? __ffs(stops) - 1 : 32;
+                unsigned long long c = 0;
+                if (lane < at) c = (v0 & VAL) + (v1 & VAL);
+                if (lane == at) c = (s0 ? v0 & VAL : 0ull) + (s0 == 1 && s1 ? v1 & VAL : 0ull);
 #pragma unroll
-                for (int j = 0; j < LB_WIDE; ++j) v[j] = p - j >= 0 ? lb_load(w + p - j) : 0ull;
-                int used = 0;
-                bool open = true, found = false;
-#pragma unroll
-                for (int j = 0; j < LB_WIDE; ++j) {
-                    open = open && !found && (v[j] >> 62) != 0ull;
-                    if (open) {
-                        base += v[j] & VAL;
-                        found = (v[j] >> 62) == 2ull;
-                        ++used;
-                    }
+                for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+                base += c;
+                if (at == 32) {
+                    p -= 64;
+                    continue;
                 }
-                if (found) break;
-                p -= used;
-                if (used == 0 && ++polls > LB_WAIT_LIMIT) {
-                    bad = 1;
+                const int a0 = __shfl_sync(0xffffffffu, s0, at), a1 = __shfl_sync(0xffffffffu, s1, at);
+                if (a0 == 2 || (a0 == 1 && a1 == 2)) break;
+                p -= 2 * at + (a0 == 1 ? 1 : 0);  // the unwritten word is read again
+                if (++polls > LB_WAIT_LIMIT) {
+                    bad = true;
                     break;
                 }
             }
-            if (!bad && chunk > 0) {
-                const unsigned long long incl = (2ull << 62) | (base + tot);
-                asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w + chunk), "l"(incl)
-                             : "memory");
+            if (lane == 0) {
+                if (!bad && chunk > 0) emit_store(w + chunk, 2ull << 62 | (base + tot));
+                s_base = base;
+                s_bad = bad;
             }
-            s_base = base;
-            s_bad = bad;
         }
         __syncthreads();
         if (s_bad) {
@@ -877,9 +896,9 @@ int launch_bin_sort(const unigs_plan& p, void* ws, cudaStream_t st) {
     cudaMemsetAsync(ss, 0, sizeof(SortState), st);
     {
         const int64_t items = (int64_t)RS_THREADS * rs_per(total);
-        // 16 pairs per thread: each block adds up to 1024 counts to the same
+        // 8 pairs per thread: each block adds up to 1024 counts to the same
         // words at its end
-        const int64_t blocks = (total + 8191) / 8192, cap = (int64_t)sm_count() * 4;
+        const int64_t blocks = (total + 4095) / 4096, cap = (int64_t)sm_count() * 4;
         depth_hist_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 512, 0, st>>>(
             touched, zbits, total, ss, words, (total + items - 1) / items * 256, emit_words,
             (total + 255) / 256, ranges, p.n_tiles);

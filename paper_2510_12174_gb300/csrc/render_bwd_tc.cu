@@ -140,15 +140,17 @@ __device__ __forceinline__ void btc_wait(uint64_t* bar, uint32_t parity, bool& t
 
 template <int NS>
 __device__ __forceinline__ void btc_stage(const BwdTcParams& P, BwdTcSmem<NS>& S, int buf,
-                                          int slot, uint32_t first, int count, int cam) {
-    // executed by the staging warp
+                                          int slot, uint32_t id, int count, int cam) {
+    // executed by the staging warp; id: the index of Gaussian `lane`
     const int lane = threadIdx.x & 31;
     const uint32_t row_bytes = (uint32_t)(P.n_sem * 2);
     const uint32_t per = REC_FLOATS * 4 + (P.sem_bulk ? row_bytes : 0u);
     if (lane == 0) mbar_expect_tx(&S.bar[buf], per * (uint32_t)count);
     __syncwarp();
-    for (int i = lane; i < count; i += 32) {
-        const uint32_t g = P.vals[first + i];
+    static_assert(BTC_BATCH <= 32, "one Gaussian per lane");
+    if (lane < count) {
+        const int i = lane;
+        const uint32_t g = id;
         S.ids[slot][i] = g;
         const size_t r = (size_t)cam * (size_t)P.n + g;
         bulk_g2s(&S.rec[buf][i][0], P.rec + r * REC_FLOATS, REC_FLOATS * 4, &S.bar[buf]);
@@ -341,6 +343,12 @@ __global__ void __launch_bounds__(BTC_THREADS, BTC_CTAS_PER_SM)
                 }
                 if (bf) ++c2b; else ++c2a;
             };
+            // index of Gaussian `lane` of the next batch, read ahead
+            auto read_id = [&](int b) -> uint32_t {
+                const int i = b * B + lane;
+                return lane < B && b >= 0 && i < n_items ? P.vals[range.x + (uint32_t)i] : 0u;
+            };
+            uint32_t id = read_id(n_batches - 1);
             for (int it = 0; it < n_batches; ++it) {
                 const int b = n_batches - 1 - it;
                 const uint32_t gk = gb0 + (uint32_t)it;
@@ -353,8 +361,8 @@ __global__ void __launch_bounds__(BTC_THREADS, BTC_CTAS_PER_SM)
                     break;
                 }
                 const int count = min(B, n_items - b * B);
-                btc_stage<NS>(P, S, bf, (int)(gk & 3u), range.x + (uint32_t)(b * B), count,
-                              cam_idx);
+                btc_stage<NS>(P, S, bf, (int)(gk & 3u), id, count, cam_idx);
+                id = read_id(b - 1);
                 btc_wait(&S.bar[bf], (gk >> 1) & 1u, timed_out);
                 if (__any_sync(0xffffffffu, timed_out)) {
                     timed_out = true;

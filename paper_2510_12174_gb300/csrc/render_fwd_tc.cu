@@ -98,7 +98,8 @@ __device__ __forceinline__ void ftc_wait(uint64_t* bar, uint32_t parity, bool& t
 // Starts the copies of a batch (count 0: an empty batch); the staging warp.
 template <int NS, int B, bool F32>
 __device__ __forceinline__ void ftc_stage(const FwdTcParams& P, FwdTcSmem<NS, B, F32>& S, int buf,
-                                          uint32_t first, int count, bool last, int cam) {
+                                          uint32_t first, int count, bool last, int cam,
+                                          uint32_t id) {
     using SemT = typename FwdTcSmem<NS, B, F32>::SemT;
     const int lane = threadIdx.x & 31;
     const uint32_t row_bytes = (uint32_t)(P.n_sem * sizeof(SemT));
@@ -106,7 +107,8 @@ __device__ __forceinline__ void ftc_stage(const FwdTcParams& P, FwdTcSmem<NS, B,
     if (lane == 0 && count > 0) mbar_expect_tx(&S.bar[buf], per * (uint32_t)count);
     __syncwarp();
     for (int i = lane; i < count; i += 32) {
-        const uint32_t g = P.vals[first + i];
+        // the first 32 indices were read a batch ahead
+        const uint32_t g = i < 32 ? id : P.vals[first + i];
         const size_t r = (size_t)cam * (size_t)P.n + g;
         bulk_g2s(&S.rec[buf][i][0], P.rec + r * REC_FLOATS, REC_FLOATS * 4, &S.bar[buf]);
         const SemT* src = static_cast<const SemT*>(P.sem) + (size_t)g * P.n_sem;
@@ -265,6 +267,9 @@ __global__ void __launch_bounds__(FTC_THREADS, (B <= 16 ? 4 : 2))
                 ++commits;
             };
             bool stop = false, empty = false;
+            constexpr int BL = B < 32 ? B : 32;
+            // index of Gaussian `lane` of the next batch, read ahead
+            uint32_t id = lane < BL && lane < n_items ? P.vals[range.x + lane] : 0u;
             for (int b = 0; b < n_batches; ++b, ++gk) {
                 const int bf = (int)(gk & 1u);
                 // the buffer's batch before last: its warps are done (waited for
@@ -277,7 +282,11 @@ __global__ void __launch_bounds__(FTC_THREADS, (B <= 16 ? 4 : 2))
                 empty = stop;
                 const bool last = stop || b + 1 == n_batches;
                 ftc_stage<NS, B, F32>(P, S, bf, range.x + (uint32_t)(b * B),
-                                      empty ? 0 : min(B, n_items - b * B), last, cam_idx);
+                                      empty ? 0 : min(B, n_items - b * B), last, cam_idx, id);
+                {
+                    const int nx = (b + 1) * B + lane;
+                    if (lane < BL && nx < n_items) id = P.vals[range.x + (uint32_t)nx];
+                }
                 if (!empty) {
                     ftc_wait(&S.bar[bf], (gk >> 1) & 1u, timed_out);
                     if (__any_sync(0xffffffffu, timed_out)) {
