@@ -599,13 +599,13 @@ __global__ void __launch_bounds__(256) emit_kernel(const EmitParams P) {
 }
 
 // The rectangles of more than MASK_TILES tiles, BIG_SEG tiles per task: a
-// warp repeats the tile test, 32 tiles per step, and takes the positions of
-// the kept ones from the pair's own counter.  (The order of a pair's
+// warp takes their bits (up to WIDE_TILES) or repeats the tile test, 32 tiles
+// per step, and the positions of the kept ones from the pair's own counter.  (The order of a pair's
 // instances does not reach the sorted lists: each lies in another tile.)
 // Task s * n_big + e is segment s of pair e; a warp's lanes look at every
 // `warps`-th task for those that exist, so that neighbouring tasks (the
 // largest rectangles stand together) go to different warps.
-constexpr int BIG_SEG = 256;
+constexpr int BIG_SEG = WIDE_TILES;
 __global__ void __launch_bounds__(256) emit_big_kernel(const EmitParams P, int max_segs) {
     __shared__ uint32_t hist[TILE_PASSES_MAX][RS_BINS];
     const int lane = threadIdx.x & 31;
@@ -645,7 +645,15 @@ __global__ void __launch_bounds__(256) emit_big_kernel(const EmitParams P, int m
             const float4* cs = reinterpret_cast<const float4*>(P.cull + (size_t)bt * CULL_FLOATS);
             const float4 c0 = cs[0], c1 = cs[1];
             const float cr[CULL_FLOATS] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-            const CullTest ct = cull_test(cr);
+            const bool wide = __shfl_sync(0xffffffffu, nt, src) <= WIDE_TILES;
+            // a test record, or the kept tiles as bits: word i in lane i
+            CullTest ct = {};
+            uint32_t bits = 0;
+            if (wide)
+                bits = lane < CULL_FLOATS
+                           ? reinterpret_cast<const uint32_t*>(cs)[lane] : 0u;
+            else
+                ct = cull_test(cr);
             const int bx0 = __shfl_sync(0xffffffffu, x0, src);
             const int by0 = __shfl_sync(0xffffffffu, y0, src);
             const int bbw = __shfl_sync(0xffffffffu, bw, src);
@@ -654,16 +662,25 @@ __global__ void __launch_bounds__(256) emit_big_kernel(const EmitParams P, int m
             const uint32_t bo = __shfl_sync(0xffffffffu, o, src);
             const uint32_t bc = __shfl_sync(0xffffffffu, cnt, src);
             uint32_t* cursor = &P.big[__shfl_sync(0xffffffffu, e, src)].w;
+            uint32_t run = 0;  // instances of a wide rectangle so far: one segment, one warp
             for (int j0 = j1; j0 < bn; j0 += 32) {
                 const int j = j0 + lane;
                 const int ry = j / bbw;
                 const int tx = bx0 + (j - ry * bbw), ty = by0 + ry;
-                const bool keep = j < bn && tile_keep(ct, tx, ty, P.tw, P.th);
-                const unsigned m = __ballot_sync(0xffffffffu, keep);
+                const unsigned m =
+                    wide ? __shfl_sync(0xffffffffu, bits, j0 / 32)
+                         : __ballot_sync(0xffffffffu,
+                                         j < bn && tile_keep(ct, tx, ty, P.tw, P.th));
+                const bool keep = (m >> lane) & 1u;
                 if (!m) continue;
-                uint32_t pos = 0;
-                if (lane == 0) pos = atomicAdd(cursor, (uint32_t)__popc(m));
-                pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m & ((1u << lane) - 1u));
+                uint32_t pos = run;
+                if (wide) {
+                    run += __popc(m);
+                } else {
+                    if (lane == 0) pos = atomicAdd(cursor, (uint32_t)__popc(m));
+                    pos = __shfl_sync(0xffffffffu, pos, 0);
+                }
+                pos += __popc(m & ((1u << lane) - 1u));
                 if (keep && pos < bc)
                     put_instance(P, hist, bo + pos,
                                  (uint32_t)cam.tile_off + (uint32_t)(ty * cam.tiles_x + tx), g);

@@ -331,14 +331,20 @@ __global__ void __launch_bounds__(256)
             const int by0 = __shfl_sync(0xffffffffu, rc.y0, src);
             const int bw = __shfl_sync(0xffffffffu, rw, src);
             const int bn = __shfl_sync(0xffffffffu, nt, src);
-            uint32_t cnt = 0;
+            uint32_t cnt = 0, word = 0;
             for (int j0 = 0; j0 < bn; j0 += 32) {
                 const int j = j0 + lane;
                 const int ry = j / bw;
                 const bool keep = j < bn && tile_keep(cs, bx0 + j - ry * bw, by0 + ry, tw, th);
-                cnt += __popc(__ballot_sync(0xffffffffu, keep));
+                const uint32_t m = __ballot_sync(0xffffffffu, keep);
+                cnt += __popc(m);
+                if (lane == j0 / 32) word = m;
             }
             if (lane == src) kept = cnt;
+            // up to WIDE_TILES the bits take the place of the test's record
+            if (bn <= WIDE_TILES && lane < CULL_FLOATS)
+                reinterpret_cast<uint32_t*>(
+                    cull)[(size_t)(base + (threadIdx.x & ~31) + src) * CULL_FLOATS + lane] = word;
         }
         // the pairs with a kept tile go to the splat setup, appended warp by
         // warp (one atomic per warp) so that its warps run full
@@ -363,7 +369,7 @@ __global__ void __launch_bounds__(256)
         zbits[t] = __float_as_uint(rc.pz);
         if (nt <= MASK_TILES) {
             masks[t] = mask;
-        } else {
+        } else if (nt > WIDE_TILES) {
             float4* cdst = reinterpret_cast<float4*>(cull + (size_t)t * CULL_FLOATS);
             cdst[0] = make_float4(cr[0], cr[1], cr[2], cr[3]);
             cdst[1] = make_float4(cr[4], cr[5], cr[6], cr[7]);
@@ -375,7 +381,7 @@ __global__ void __launch_bounds__(256)
 // appended): the double-float conic and centre, the principal axes, the SH
 // colour and the ray-ellipsoid record.  The binning recipe is recomputed (the
 // same bits as in the culling pass) for the rotation, depth and radius.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 3)
     preprocess_splat_kernel(const unigs_gaussians g, const CamTable* __restrict__ tab,
                             float lowpass, const uint32_t* __restrict__ kept_list,
                             const WsHeader* __restrict__ hdr, float* __restrict__ rec,
@@ -434,10 +440,26 @@ __global__ void __launch_bounds__(256)
         sh_eval_basis(dx, dy, dz, deg, Y);
         float col[3] = {0.5f, 0.5f, 0.5f};
         const size_t shb = (size_t)i * n_sh * 3;
-        for (int kk = 0; kk < n_sh; ++kk)
+        if (deg & 1) {
+            // 4 or 16 coefficients: rows of whole 16-byte (bfloat16: 8-byte) words
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch)
-                col[ch] = fmaf(Y[kk], load_feat(g.sh, shb + kk * 3 + ch, g.feat_dtype), col[ch]);
+            for (int k0 = 0; k0 < 16; k0 += 4) {
+                if (k0 >= n_sh) break;
+                float hc[12];
+                load_feats<12>(g.sh, shb + 3 * k0, g.feat_dtype, hc);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int ch = 0; ch < 3; ++ch)
+                        col[ch] = fmaf(Y[k0 + e], hc[3 * e + ch], col[ch]);
+            }
+        } else {
+            for (int kk = 0; kk < n_sh; ++kk)
+#pragma unroll
+                for (int ch = 0; ch < 3; ++ch)
+                    col[ch] = fmaf(Y[kk], load_feat(g.sh, shb + kk * 3 + ch, g.feat_dtype),
+                                   col[ch]);
+        }
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) o[R_RGB + ch] = fmaxf(col[ch], 0.f);
 

@@ -526,13 +526,22 @@ __global__ void __launch_bounds__(PREBWD_THREADS, 4) preprocess_bwd_kernel(const
                     sh_eval_basis_grad(d[0], d[1], d[2], DEG, dY);
                     float g_dir[3] = {0.f, 0.f, 0.f};
                     const size_t shb = (size_t)i * n_sh * 3;
+                    // rows of 4 or 16 coefficients are whole words: 3 or 12 vector
+                    // loads, where an element per load cost a sector each
+                    float hv[3 * n_sh];
+                    if constexpr (3 * n_sh % 4 == 0)
+                        load_feats<3 * n_sh>(P.g.sh, shb, P.g.feat_dtype, hv);
+                    else
+#pragma unroll
+                        for (int e = 0; e < 3 * n_sh; ++e)
+                            hv[e] = load_feat(P.g.sh, shb + e, P.g.feat_dtype);
 #pragma unroll
                     for (int ch = 0; ch < 3; ++ch) {
                         float hc[n_sh];
                         float raw = 0.5f;
 #pragma unroll
                         for (int kk = 0; kk < n_sh; ++kk) {
-                            hc[kk] = load_feat(P.g.sh, shb + kk * 3 + ch, P.g.feat_dtype);
+                            hc[kk] = hv[3 * kk + ch];
                             raw = fmaf(Y[kk], hc[kk], raw);
                         }
                         if (raw < 0.f) continue;  // clamped at 0
@@ -699,11 +708,6 @@ __global__ void __launch_bounds__(PREBWD_THREADS, 4) preprocess_bwd_kernel(const
                 for (int b = 0; b < 3; ++b) g_R[a][b] = row[3 + 3 * a + b];
             }
             const float g_op = row[18], g_k = row[19];
-            float g_sh[n_sh][3];
-#pragma unroll
-            for (int kk = 0; kk < n_sh; ++kk)
-#pragma unroll
-                for (int ch = 0; ch < 3; ++ch) g_sh[kk][ch] = row[20 + 3 * kk + ch];
             // the rotation's local-frame gradient as a matrix gradient:
             // 1/2 R [g_theta]_x has the same derivative along every tangent R [e]_x
             {
@@ -738,12 +742,18 @@ __global__ void __launch_bounds__(PREBWD_THREADS, 4) preprocess_bwd_kernel(const
             for (int a = 0; a < 4; ++a) PUT(O.quat, a * n + i, g_q[a]);
             PUT(O.opacity, i, g_op);
             PUT(O.kfac, i, g_k);
-#pragma unroll
-            for (int kk = 0; kk < n_sh; ++kk)
-#pragma unroll
-                for (int ch = 0; ch < 3; ++ch) PUT(O.sh, ((size_t)i * n_sh + kk) * 3 + ch, g_sh[kk][ch]);
-#undef PUT
         }
+        // the SH gradients of the warp's Gaussians are consecutive in memory:
+        // stored from the accumulator rows by consecutive lanes
+        if (P.out.sh) {
+            const int left = n - g0 < 32 ? (int)(n - g0) : 32;
+            float* dst = P.out.sh + (size_t)g0 * (3 * n_sh);
+            for (int e = lane; e < left * 3 * n_sh; e += 32) {
+                const float v = acc[e / (3 * n_sh) * ACCS + 20 + e % (3 * n_sh)];
+                dst[e] = P.out.accumulate ? dst[e] + v : v;
+            }
+        }
+#undef PUT
         // the rows are rewritten for the next 32 Gaussians only after every
         // lane has read its own
         __syncwarp();

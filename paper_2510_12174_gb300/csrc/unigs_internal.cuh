@@ -238,10 +238,12 @@ __device__ __forceinline__ bool tile_keep(const CullTest& c, int tx, int ty, int
 
 constexpr int SCAN_ITEMS = 4096;   // elements per scan block (256 threads x 16)
 constexpr int LOSS_MAX_BLOCKS = 2048;  // block partials of the loss reduction
-// Rectangles of at most this many tiles carry a bit mask of their kept tiles
-// from the preprocess to the emission, which then repeats no tile test; larger
-// ones (rare) carry the test's record.
+// Rectangles of at most MASK_TILES tiles carry a bit mask of their kept tiles
+// from the preprocess to the emission, those of at most WIDE_TILES one in the
+// place of the test's record (8 words); the emission repeats the tile test for
+// larger ones only.
 constexpr int MASK_TILES = 64;
+constexpr int WIDE_TILES = 32 * CULL_FLOATS;
 constexpr int SORT_ITEMS = 2048;   // keys per block of the 64-bit pair sort (256 threads x 8)
 // Blocks of the single-kernel radix passes: RS_THREADS threads (one per digit
 // value at most) of RS_PER keys.
@@ -299,6 +301,36 @@ __device__ inline void set_status(WsHeader* h, uint32_t code) {
 __device__ __forceinline__ float load_feat(const void* base, size_t i, int bf16) {
     if (bf16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(base)[i]);
     return reinterpret_cast<const float*>(base)[i];
+}
+
+// N consecutive features from element i0 on, N and i0 multiples of 4 and base
+// 16-byte aligned: 16 (float32) or 8 (bfloat16) bytes a load.
+template <int N>
+__device__ __forceinline__ void load_feats(const void* base, size_t i0, int bf16, float (&h)[N]) {
+    static_assert(N % 4 == 0, "whole vectors");
+    if (bf16) {
+        const uint2* src = reinterpret_cast<const uint2*>(
+            reinterpret_cast<const __nv_bfloat16*>(base) + i0);
+#pragma unroll
+        for (int q = 0; q < N / 4; ++q) {
+            const uint2 v = src[q];
+            h[4 * q] = __uint_as_float(v.x << 16);
+            h[4 * q + 1] = __uint_as_float(v.x & 0xffff0000u);
+            h[4 * q + 2] = __uint_as_float(v.y << 16);
+            h[4 * q + 3] = __uint_as_float(v.y & 0xffff0000u);
+        }
+    } else {
+        const float4* src = reinterpret_cast<const float4*>(
+            reinterpret_cast<const float*>(base) + i0);
+#pragma unroll
+        for (int q = 0; q < N / 4; ++q) {
+            const float4 v = src[q];
+            h[4 * q] = v.x;
+            h[4 * q + 1] = v.y;
+            h[4 * q + 2] = v.z;
+            h[4 * q + 3] = v.w;
+        }
+    }
 }
 
 // ----------------------------------------------------------------------------
