@@ -457,11 +457,10 @@ __device__ __forceinline__ void put(float* p, int64_t i, float v, int acc) {
 }
 
 // s[i][j] += sum over the tile's anchors (in order) of x[i][a] z[j][a], 4 x RJ
-// entries; with `bias` also b[i] += sum_a x[i][a].
+// entries.
 template <typename T, int RJ>
-__device__ __forceinline__ void outer_sums(const float* x, const float* z, float* s, float* b,
-                                           bool bias) {
-    float acc[4][RJ] = {}, sb[4] = {};
+__device__ __forceinline__ void outer_sums(const float* x, const float* z, float* s) {
+    float acc[4][RJ] = {};
     for (int a = 0; a < T::TA; a += 4) {
         float xv[4][4], zv[RJ][4];
 #pragma unroll
@@ -471,11 +470,9 @@ __device__ __forceinline__ void outer_sums(const float* x, const float* z, float
 #pragma unroll
         for (int e = 0; e < 4; ++e)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (bias) sb[i] += xv[i][e];
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < RJ; ++j) acc[i][j] = fmaf(xv[i][e], zv[j][e], acc[i][j]);
-            }
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -484,7 +481,22 @@ __device__ __forceinline__ void outer_sums(const float* x, const float* z, float
 #pragma unroll
         for (int j = 0; j < RJ; ++j) q[j] += acc[i][j];
         st_anchors<RJ>(s + i * WS, q);
-        if (bias) b[i] += sb[i];
+    }
+}
+
+// b[r] += sum over the tile's anchors of x[r][a], n rows, a warp per row (in
+// the products' loop the sums cost every thread 16 additions per 32
+// multiply-adds).
+template <typename T>
+__device__ __forceinline__ void row_sums(const float* x, int n, float* b) {
+    const int lane = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < n; r += T::NT / 32) {
+        float v = 0.f;
+#pragma unroll
+        for (int a = lane; a < T::TA; a += 32) v += x[r * T::S + a];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) b[r] += v;
     }
 }
 
@@ -569,8 +581,43 @@ __device__ __forceinline__ void load_upstream(const GradIn& G, int X, int nr, in
     }
 }
 
+// Adds the parameter-gradient sums of the NC blocks of a cluster to the
+// outputs, this block's share of the entries.  One pass over the layout with
+// all NC peers' loads in flight: array by array and peer by peer, each entry
+// waited for NC remote loads in a row, half the time of a small backward.
+template <int NC, int NT>
+__device__ void add_params(const cg::cluster_group& cl, const WLayout& L, const AnchorGradOut& R,
+                           int M, float* sg) {
+    for (int e = (int)cl.block_rank() * NT + threadIdx.x; e < L.total; e += NC * NT) {
+        float v[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) v[k] = *cl.map_shared_rank(sg + e, k);
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) t += (double)v[k];
+        int X = 0;
+#pragma unroll
+        for (int x = 1; x < NMLP; ++x)
+            if (L.out[x] > 0 && e >= L.w1[x]) X = x;
+        float* dst;
+        int i = e - L.w1[X];
+        if (i < AH * AF) {
+            dst = R.w1[X] + i;
+        } else if ((i -= AH * AF) < AH) {
+            dst = R.b1[X] + i;
+        } else {
+            i -= AH;
+            const bool w2 = i < L.rows[X] * AH;
+            const int row = param_row(X, L.out[X], w2 ? i / AH : i - L.rows[X] * AH, M);
+            if (row < 0) continue;
+            dst = w2 ? R.w2[X] + row * AH + i % AH : R.b2[X] + row;
+        }
+        atomicAdd(dst, (float)t);
+    }
+}
+
 template <typename T>
-__global__ void __launch_bounds__(T::NT) anchor_decode_bwd_kernel(const AnchorIn P, const WLayout L,
+__global__ void __launch_bounds__(T::NT, 1) anchor_decode_bwd_kernel(const AnchorIn P, const WLayout L,
                                                                   const GradIn G,
                                                                   const AnchorGradOut R) {
     constexpr int S = T::S, RA = T::RA, NT = T::NT, GROUPS = T::GROUPS;
@@ -694,13 +741,13 @@ __global__ void __launch_bounds__(T::NT) anchor_decode_bwd_kernel(const AnchorIn
             for (int t = tid; t < (8 + nr / 4) * TPR; t += NT) {
                 const int row = 4 * (t / TPR), col = RJ * (t % TPR);
                 if (row < AH)
-                    outer_sums<T, RJ>(gp + row * S, ft + col * S, sg + L.w1[X] + row * WS + col,
-                                      sg + L.b1[X] + row, col == 0);
+                    outer_sums<T, RJ>(gp + row * S, ft + col * S, sg + L.w1[X] + row * WS + col);
                 else
                     outer_sums<T, RJ>(gy + (row - AH) * S, h + col * S,
-                                      sg + L.w2[X] + (row - AH) * WS + col,
-                                      sg + L.b2[X] + row - AH, col == 0);
+                                      sg + L.w2[X] + (row - AH) * WS + col);
             }
+            row_sums<T>(gp, AH, sg + L.b1[X]);
+            row_sums<T>(gy, nr, sg + L.b2[X]);
             __syncthreads();
         }
         // features, position, offsets and scale: mu_m = x + l (x) O_m
@@ -742,23 +789,10 @@ __global__ void __launch_bounds__(T::NT) anchor_decode_bwd_kernel(const AnchorIn
     // host without accumulate).
     const cg::cluster_group cl = cg::this_cluster();
     cl.sync();
-    const int nc = (int)cl.num_blocks(), first = (int)cl.block_rank() * NT + tid, step = nc * NT;
-    auto total = [&](int e) {
-        double v = 0.0;
-        for (int k = 0; k < nc; ++k) v += (double)*cl.map_shared_rank(sg + e, k);
-        return (float)v;
-    };
-    for (int X = 0; X < NMLP; ++X) {
-        if (L.out[X] == 0) continue;
-        for (int i = first; i < AH * AF; i += step) atomicAdd(R.w1[X] + i, total(L.w1[X] + i));
-        for (int i = first; i < AH; i += step) atomicAdd(R.b1[X] + i, total(L.b1[X] + i));
-        for (int i = first; i < L.rows[X] * AH; i += step) {
-            const int j = i / AH, dst = param_row(X, L.out[X], j, M);
-            if (dst < 0) continue;
-            atomicAdd(R.w2[X] + dst * AH + i % AH, total(L.w2[X] + i));
-            if (i % AH == 0) atomicAdd(R.b2[X] + dst, total(L.b2[X] + j));
-        }
-    }
+    if (cl.num_blocks() == 8)
+        add_params<8, NT>(cl, L, R, M, sg);
+    else
+        add_params<2, NT>(cl, L, R, M, sg);
     cl.sync();  // a block's shared memory stays until its peers have read it
 }
 

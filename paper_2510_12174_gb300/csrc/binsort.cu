@@ -398,6 +398,7 @@ struct EmitParams {
     const uint32_t* touched;
     const unsigned long long* masks;
     const float* cull;
+    const uint32_t* keep_bits;        // kept-tile bits of the large rectangles
     const uint32_t* order;            // kept pairs by depth
     SortState* st;
     WsHeader* hdr;
@@ -599,7 +600,7 @@ __global__ void __launch_bounds__(256) emit_kernel(const EmitParams P) {
 }
 
 // The rectangles of more than MASK_TILES tiles, BIG_SEG tiles per task: a
-// warp takes their bits (up to WIDE_TILES) or repeats the tile test, 32 tiles
+// warp takes their bits or, without them, repeats the tile test, 32 tiles
 // per step, and the positions of the kept ones from the pair's own counter.  (The order of a pair's
 // instances does not reach the sorted lists: each lies in another tile.)
 // Task s * n_big + e is segment s of pair e; a warp's lanes look at every
@@ -645,36 +646,47 @@ __global__ void __launch_bounds__(256) emit_big_kernel(const EmitParams P, int m
             const float4* cs = reinterpret_cast<const float4*>(P.cull + (size_t)bt * CULL_FLOATS);
             const float4 c0 = cs[0], c1 = cs[1];
             const float cr[CULL_FLOATS] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-            const bool wide = __shfl_sync(0xffffffffu, nt, src) <= WIDE_TILES;
-            // a test record, or the kept tiles as bits: word i in lane i
+            const int snt = __shfl_sync(0xffffffffu, nt, src);
+            const bool wide = snt <= WIDE_TILES;
+            const int j1 = __shfl_sync(0xffffffffu, seg, src) * BIG_SEG;
+            // the segment's kept tiles as bits, word i in lane i, or the test
+            const uint32_t at = wide ? 0u : __float_as_uint(cr[C_BITS]);
+            const bool known = at != NO_BITS;
+            const uint32_t* words =
+                wide ? reinterpret_cast<const uint32_t*>(cs) : P.keep_bits + (known ? at : 0u) + j1 / 32;
             CullTest ct = {};
             uint32_t bits = 0;
-            if (wide)
-                bits = lane < CULL_FLOATS
-                           ? reinterpret_cast<const uint32_t*>(cs)[lane] : 0u;
-            else
+            if (!known)
                 ct = cull_test(cr);
+            else if (lane < BIG_SEG / 32 && j1 + 32 * lane < snt)
+                bits = words[lane];
             const int bx0 = __shfl_sync(0xffffffffu, x0, src);
             const int by0 = __shfl_sync(0xffffffffu, y0, src);
             const int bbw = __shfl_sync(0xffffffffu, bw, src);
-            const int j1 = __shfl_sync(0xffffffffu, seg, src) * BIG_SEG;
-            const int bn = min(__shfl_sync(0xffffffffu, nt, src), j1 + BIG_SEG);
+            const int bn = min(snt, j1 + BIG_SEG);
             const uint32_t bo = __shfl_sync(0xffffffffu, o, src);
             const uint32_t bc = __shfl_sync(0xffffffffu, cnt, src);
             uint32_t* cursor = &P.big[__shfl_sync(0xffffffffu, e, src)].w;
-            uint32_t run = 0;  // instances of a wide rectangle so far: one segment, one warp
+            // where the bits are known, one addition reserves the segment's
+            // positions (a wide rectangle is one segment of one warp)
+            uint32_t run = 0;
+            if (known && !wide) {
+                const uint32_t total = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(bits));
+                if (lane == 0) run = atomicAdd(cursor, total);
+                run = __shfl_sync(0xffffffffu, run, 0);
+            }
             for (int j0 = j1; j0 < bn; j0 += 32) {
                 const int j = j0 + lane;
                 const int ry = j / bbw;
                 const int tx = bx0 + (j - ry * bbw), ty = by0 + ry;
                 const unsigned m =
-                    wide ? __shfl_sync(0xffffffffu, bits, j0 / 32)
+                    known ? __shfl_sync(0xffffffffu, bits, (j0 - j1) / 32)
                          : __ballot_sync(0xffffffffu,
                                          j < bn && tile_keep(ct, tx, ty, P.tw, P.th));
                 const bool keep = (m >> lane) & 1u;
                 if (!m) continue;
                 uint32_t pos = run;
-                if (wide) {
+                if (known) {
                     run += __popc(m);
                 } else {
                     if (lane == 0) pos = atomicAdd(cursor, (uint32_t)__popc(m));
@@ -965,6 +977,7 @@ int launch_bin_sort(const unigs_plan& p, void* ws, cudaStream_t st) {
         E.touched = touched;
         E.masks = cull_masks(ws, p);
         E.cull = cull_records(ws, p);
+        E.keep_bits = cull_bits(ws, p);
         E.order = dt[1];
         E.st = ss;
         E.hdr = hdr;

@@ -230,7 +230,8 @@ unigs_status unigs_plan_init(unigs_plan* plan, const unigs_gaussians* g, const u
     // (the binning's depth sort borrows up to 112 bytes a pair of it)
     sizes[OFF_GREC] = sizeof(double) * GREC_FLOATS * (size_t)total;
     sizes[OFF_CULL] = sizeof(float) * CULL_FLOATS * (size_t)total +
-                      sizeof(unsigned long long) * (size_t)(total + 1);
+                      sizeof(unsigned long long) * (size_t)(total + 1) +
+                      sizeof(uint32_t) * (size_t)bit_word_count(cap);
     // float32 copy of bfloat16 semantic rows, refreshed by every preprocess
     // when an FP32-pipe composite will read it
     sizes[OFF_SEM32] = sem32_needed(*plan) ? sizeof(float) * (size_t)g->n * g->n_sem : 0;

@@ -233,7 +233,7 @@ __device__ __forceinline__ void cull_record(const Recipe& rc, float op, float* c
     const float ac = __fadd_rn(rc.a, rc.c);
     cr[C_NOCULL] = (__fmul_rn(ac, ac) > __fmul_rn(4096.f, rc.det)) ? 1.f : 0.f;
     cr[C_QLIM] = cull_qlim(op);
-    cr[7] = 0.f;
+    cr[C_BITS] = __uint_as_float(NO_BITS);
 }
 
 // Shares lane src's test record and rectangle with the warp.
@@ -250,6 +250,7 @@ __global__ void __launch_bounds__(256)
                       int tw, int th, float lowpass, uint2* __restrict__ rect,
                       uint32_t* __restrict__ touched, uint32_t* __restrict__ zbits,
                       unsigned long long* __restrict__ masks, float* __restrict__ cull,
+                      uint32_t* __restrict__ bits, int64_t n_bit_words,
                       WsHeader* __restrict__ hdr, uint32_t* __restrict__ kept_list) {
     const int64_t n = g.n;
     const int64_t total = n * (int64_t)n_cams;
@@ -331,6 +332,23 @@ __global__ void __launch_bounds__(256)
             const int by0 = __shfl_sync(0xffffffffu, rc.y0, src);
             const int bw = __shfl_sync(0xffffffffu, rw, src);
             const int bn = __shfl_sync(0xffffffffu, nt, src);
+            // the kept tiles as bits: up to WIDE_TILES in the place of the
+            // test's record, else in the common array where words are left
+            const int words = (bn + 31) / 32;
+            uint32_t* dst = nullptr;
+            uint32_t at = NO_BITS;
+            if (bn <= WIDE_TILES) {
+                dst = reinterpret_cast<uint32_t*>(cull) +
+                      (size_t)(base + (threadIdx.x & ~31) + src) * CULL_FLOATS;
+            } else {
+                unsigned long long first = 0;
+                if (lane == 0) first = atomicAdd(&hdr->bit_words, (unsigned long long)words);
+                first = __shfl_sync(0xffffffffu, first, 0);
+                if (first + words <= (unsigned long long)n_bit_words && first + words < NO_BITS) {
+                    at = (uint32_t)first;
+                    dst = bits + first;
+                }
+            }
             uint32_t cnt = 0, word = 0;
             for (int j0 = 0; j0 < bn; j0 += 32) {
                 const int j = j0 + lane;
@@ -338,13 +356,16 @@ __global__ void __launch_bounds__(256)
                 const bool keep = j < bn && tile_keep(cs, bx0 + j - ry * bw, by0 + ry, tw, th);
                 const uint32_t m = __ballot_sync(0xffffffffu, keep);
                 cnt += __popc(m);
-                if (lane == j0 / 32) word = m;
+                // 32 words at a time
+                const int w = j0 / 32;
+                if (lane == (w & 31)) word = m;
+                if (dst && ((w & 31) == 31 || w + 1 == words) && lane <= (w & 31))
+                    dst[(w & ~31) + lane] = word;
             }
-            if (lane == src) kept = cnt;
-            // up to WIDE_TILES the bits take the place of the test's record
-            if (bn <= WIDE_TILES && lane < CULL_FLOATS)
-                reinterpret_cast<uint32_t*>(
-                    cull)[(size_t)(base + (threadIdx.x & ~31) + src) * CULL_FLOATS + lane] = word;
+            if (lane == src) {
+                kept = cnt;
+                cr[C_BITS] = __uint_as_float(at);
+            }
         }
         // the pairs with a kept tile go to the splat setup, appended warp by
         // warp (one atomic per warp) so that its warps run full
@@ -541,6 +562,7 @@ __global__ void init_kernel(CamTable tab, int n_cams, CamTable* __restrict__ dst
         hdr->n_blend = 0;
         hdr->nonfinite = 0;
         hdr->n_kept = 0;
+        hdr->bit_words = 0;
     }
 }
 
@@ -617,8 +639,8 @@ int launch_preprocess(const unigs_plan& p, const unigs_gaussians& g, const CamTa
         preprocess_kernel<<<grid, 256, 0, st>>>(
             g, ws_ptr<CamTable>(ws, p, OFF_CAM), p.n_cams, p.cfg.tile_w, p.cfg.tile_h,
             p.cfg.lowpass, ws_ptr<uint2>(ws, p, OFF_RECT), ws_ptr<uint32_t>(ws, p, OFF_TOUCH),
-            ws_ptr<uint32_t>(ws, p, OFF_ZBITS), cull_masks(ws, p), cull_records(ws, p), hdr,
-            kept_list);
+            ws_ptr<uint32_t>(ws, p, OFF_ZBITS), cull_masks(ws, p), cull_records(ws, p),
+            cull_bits(ws, p), bit_word_count(p.capacity), hdr, kept_list);
         // grid-stride over the list, whose length only the device knows
         const int64_t cap2 = (int64_t)sm_count() * 32;
         const int grid2 = (int)(blocks < cap2 ? blocks : cap2);

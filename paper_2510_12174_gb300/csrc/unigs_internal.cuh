@@ -159,7 +159,9 @@ struct WsHeader {
     uint32_t work_bwd;
     uint32_t nonfinite;          // first parameter array found non-finite (flag set)
     uint32_t n_kept;             // (camera, Gaussian) pairs with a kept tile (preprocess)
-    uint32_t pad[52];
+    uint32_t pad0;
+    unsigned long long bit_words;  // words of the kept-tile bits in use (preprocess)
+    uint32_t pad[48];
 };
 static_assert(sizeof(WsHeader) == 256, "WsHeader layout");
 
@@ -172,8 +174,9 @@ enum {
 static_assert(OFF_END <= 20, "unigs_plan::off holds 20 region offsets");
 
 // Per-(camera, Gaussian) record of the opacity-aware tile test (8 floats):
-// float32 projected centre, float32 conic (kA, kB, kC), qlim, no-cull flag.
-enum { C_MX = 0, C_MY, C_KA, C_KB, C_KC, C_QLIM, C_NOCULL, CULL_FLOATS = 8 };
+// float32 projected centre, float32 conic (kA, kB, kC), qlim, no-cull flag,
+// and the first word of the kept-tile bits (as bits; NO_BITS: none).
+enum { C_MX = 0, C_MY, C_KA, C_KB, C_KC, C_QLIM, C_NOCULL, C_BITS, CULL_FLOATS = 8 };
 
 // Opacity-aware tile test, float32 recipe with non-contractible operations
 // (identical operation order in the oracle's binning): keep the tile when the
@@ -240,8 +243,9 @@ constexpr int SCAN_ITEMS = 4096;   // elements per scan block (256 threads x 16)
 constexpr int LOSS_MAX_BLOCKS = 2048;  // block partials of the loss reduction
 // Rectangles of at most MASK_TILES tiles carry a bit mask of their kept tiles
 // from the preprocess to the emission, those of at most WIDE_TILES one in the
-// place of the test's record (8 words); the emission repeats the tile test for
-// larger ones only.
+// place of the test's record (8 words), larger ones a place in a common array
+// of words (record [7], C_BITS) while it lasts: only rectangles that found it
+// full are tested again.
 constexpr int MASK_TILES = 64;
 constexpr int WIDE_TILES = 32 * CULL_FLOATS;
 constexpr int SORT_ITEMS = 2048;   // keys per block of the 64-bit pair sort (256 threads x 8)
@@ -282,6 +286,15 @@ __host__ inline unsigned long long* cull_masks(void* ws, const unigs_plan& p) {
 __host__ inline float* cull_records(void* ws, const unigs_plan& p) {
     const size_t total = (size_t)p.n * (size_t)p.n_cams;
     return reinterpret_cast<float*>(cull_masks(ws, p) + (total + 1) / 2 * 2);
+}
+
+// Words of kept-tile bits: 4 bits per instance of the capacity (a rectangle's
+// tiles are a few times its kept ones).
+constexpr uint32_t NO_BITS = 0xffffffffu;
+__host__ inline int64_t bit_word_count(int64_t capacity) { return capacity / 8 + 1024; }
+__host__ inline uint32_t* cull_bits(void* ws, const unigs_plan& p) {
+    const size_t total = (size_t)p.n * (size_t)p.n_cams;
+    return reinterpret_cast<uint32_t*>(cull_records(ws, p) + total * CULL_FLOATS);
 }
 
 __device__ inline const DevCam& cam_of_tile(const CamTable* tab, int n_cams, int64_t gtile,
