@@ -64,16 +64,18 @@ struct BwdSmem {
     // 16-byte chunk k of row p is stored at chunk k ^ (p % (NS / 4)), so both
     // the per-thread row reads and the per-row channel gathers of a warp are
     // free of bank conflicts without padding
-    float rec[2][B][REC_FLOATS];
-    float sem[2][B][NS];
+    // staged batches: a warp runs up to NB - 1 of them ahead of the slowest
+    static constexpr int NB = B == 8 && NS <= 32 ? 8 : 2;
+    float rec[NB][B][REC_FLOATS];
+    float sem[NB][B][NS];
     float gO[TILE_PIX * NS];
     float2 wv[8][32];  // per warp: (w, w) of its pixels for the current Gaussian
-    uint32_t ids[2][B];
-    uint64_t bar[2];   // batch staged (bulk bytes + the producer warp's arrival)
-    uint64_t cons[2];  // batch consumed (one arrival per warp)
+    uint32_t ids[NB][B];
+    uint64_t bar[NB];   // batch staged (bulk bytes + the producer warp's arrival)
+    uint64_t cons[NB];  // batch consumed (one arrival per warp)
     uint32_t max_last;
     int tile;
-    uint32_t issued[2];  // staging phases started per buffer (one thread counts)
+    uint32_t issued[NB];  // staging phases started per buffer (one thread counts)
 };
 
 // Offset of channel c of pixel row p in the swizzled upstream-gradient tile.
@@ -157,18 +159,19 @@ template <int NS, int B>
 __global__ void __launch_bounds__(256, (B <= 8 ? 3 : 2)) render_bwd_kernel(const BwdParams P) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     BwdSmem<NS, B>& S = *reinterpret_cast<BwdSmem<NS, B>*>(smem_raw);
+    constexpr uint32_t NB = BwdSmem<NS, B>::NB;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     // once per CTA: init barriers, zero the semantic padding
     if (tid == 0) {
-        mbar_init(&S.bar[0], 1);
-        mbar_init(&S.bar[1], 1);
-        mbar_init(&S.cons[0], 8);
-        mbar_init(&S.cons[1], 8);
+        for (int b = 0; b < NB; ++b) {
+            mbar_init(&S.bar[b], 1);
+            mbar_init(&S.cons[b], 8);
+            S.issued[b] = 0u;
+        }
         fence_mbar_init();
-        S.issued[0] = S.issued[1] = 0u;
     }
-    for (int j = tid; j < 2 * B * NS; j += 256) (&S.sem[0][0][0])[j] = 0.f;
+    for (int j = tid; j < NB * B * NS; j += 256) (&S.sem[0][0][0])[j] = 0.f;
     // the upstream-gradient rows are addressed by XOR within a row, which
     // needs the tile aligned to the row size (it sits at a multiple of 256
     // bytes of the dynamic shared memory, whose start is so aligned)
@@ -179,9 +182,9 @@ __global__ void __launch_bounds__(256, (B <= 8 ? 3 : 2)) render_bwd_kernel(const
     }
     const uint32_t a_row = go_row<NS>(go_base, tid);
     __syncthreads();
-    // per buffer: phases of bar[] waited for and consumptions (uniform across
-    // the CTA); scalars, so that they stay in registers
-    uint32_t loads0 = 0u, loads1 = 0u, used0 = 0u, used1 = 0u;
+    // batches begun by this CTA (uniform) and staged by warp 0: batch gk uses
+    // buffer gk % NB and is phase gk / NB of the buffer's barriers
+    uint32_t gk = 0u, gs = 0u;
     bool timed_out = false;
 
     for (;;) {
@@ -236,35 +239,49 @@ __global__ void __launch_bounds__(256, (B <= 8 ? 3 : 2)) render_bwd_kernel(const
         const int n_items = (int)S.max_last;
         const int n_batches = (n_items + B - 1) / B;
         const uint2 range = P.ranges[gtile];
-        // Staging pipeline: warp 0 stages batch it+1 while every warp composites
-        // batch it; a buffer is restaged only after all 8 warps have arrived on
-        // its "consumed" barrier, so the warps never meet at a CTA barrier
-        // inside the tile.
+        // Staging pipeline: before each of its batches warp 0 stages as many of
+        // the next ones as have a free buffer (one that all 8 warps have
+        // arrived for on its "consumed" barrier) and waits for a buffer only
+        // for the batch it needs itself, so the warps never meet at a CTA
+        // barrier inside the tile.  Eight buffers of 8 Gaussians (where they
+        // fit) let a warp run ahead of the slowest: the backward of 200k
+        // Gaussians at 640x480 takes 0.526 ms, with two 0.540 ms.
         // Warp 0 restages a buffer only if none of its own waits gave up (a
-        // warp-uniform decision): it waits on every staging phase itself, so
-        // the buffer's previous copy was seen to land and at most one copy
-        // per buffer is ever in flight; the exit drain finds it by S.issued.
-        auto produce = [&](int bf, uint32_t first, int cnt) {
-            const uint32_t u = bf ? used1 : used0;
-            if (u > 0 && !mbar_wait_bounded(&S.cons[bf], (u - 1) & 1u, BWAIT_LIMIT))
-                timed_out = true;
-            if (__any_sync(0xffffffffu, timed_out)) return;
-            bwd_issue<NS, B>(P, S, bf, first, cnt, cam_idx);
-            if (lane == 0) ++S.issued[bf];
+        // warp-uniform decision): the buffer's previous copy was waited for by
+        // every warp before it arrived, so at most one copy per buffer is ever
+        // in flight; the exit drain finds it by S.issued.
+        const uint32_t gk0 = gk, gk_end = gk + (uint32_t)n_batches;
+        auto stage_ahead = [&]() {
+            while (gs < gk_end && gs < gk + NB) {
+                const uint32_t bf = gs % NB, ph = gs / NB;
+                if (ph > 0) {
+                    if (gs == gk) {
+                        if (!mbar_wait_bounded(&S.cons[bf], (ph - 1) & 1u, BWAIT_LIMIT))
+                            timed_out = true;
+                        if (__any_sync(0xffffffffu, timed_out)) timed_out = true;
+                    } else if (!__all_sync(0xffffffffu, mbar_test(&S.cons[bf], (ph - 1) & 1u))) {
+                        return;
+                    }
+                }
+                if (timed_out) return;
+                const int b = n_batches - 1 - (int)(gs - gk0);
+                bwd_issue<NS, B>(P, S, (int)bf, range.x + (uint32_t)(b * B),
+                                 min(B, n_items - b * B), cam_idx);
+                if (lane == 0) ++S.issued[bf];
+                ++gs;
+            }
         };
-        if (warp == 0 && n_batches > 0)
-            produce(0, range.x + (n_batches - 1) * B, min(B, n_items - (n_batches - 1) * B));
 
         float Sacc = 0.f;  // sum over already processed (later) Gaussians of w_j G_j
-        for (int it = 0; it < n_batches; ++it) {
+        for (int it = 0; it < n_batches; ++it, ++gk) {
             const int b = n_batches - 1 - it;
-            const int buf = it & 1;
-            if (warp == 0 && b > 0) produce(buf ^ 1, range.x + (b - 1) * B, B);
-            {
-                const uint32_t ph = buf ? loads1 : loads0;
-                if (!mbar_wait_bounded(&S.bar[buf], ph & 1u, BWAIT_LIMIT)) timed_out = true;
-                if (buf) ++loads1; else ++loads0;
+            const int buf = (int)(gk % NB);
+            if (warp == 0) {
+                if (__any_sync(0xffffffffu, timed_out)) timed_out = true;
+                stage_ahead();
             }
+            if (!timed_out && !mbar_wait_bounded(&S.bar[buf], (gk / NB) & 1u, BWAIT_LIMIT))
+                timed_out = true;
             const int count = min(B, n_items - b * B);
             if (!__all_sync(0xffffffffu, timed_out) && (uint32_t)(b * B) < wlast) {
             const int reach = min(count, (int)(wlast - (uint32_t)(b * B)));
@@ -356,14 +373,17 @@ __global__ void __launch_bounds__(256, (B <= 8 ? 3 : 2)) render_bwd_kernel(const
             // this warp is done with the batch's buffers
             __syncwarp();
             if (lane == 0) mbar_arrive(&S.cons[buf]);
-            if (buf) ++used1; else ++used0;
         }
         // a bounded wait that gave up ends the CTA (uniformly)
         if (__syncthreads_or(timed_out)) break;
     }
     // no bulk copy may still be landing in this CTA's shared memory when it
     // exits (after a timeout at most one per buffer is in flight)
-    if (tid == 0 && !drain_bulk(S.bar, S.issued[0], S.issued[1], BWAIT_LIMIT)) timed_out = true;
+    if (tid == 0)
+        for (uint32_t b = 0; b < NB; ++b)
+            if (S.issued[b] > 0 &&
+                !mbar_wait_bounded(&S.bar[b], (S.issued[b] - 1) & 1u, BWAIT_LIMIT))
+                timed_out = true;
     if (timed_out && lane == 0) set_status(P.hdr, UNIGS_ERR_TIMEOUT);
 }
 
