@@ -488,38 +488,45 @@ __global__ void __launch_bounds__(BTC_THREADS, BTC_CTAS_PER_SM)
                 if (!__all_sync(0xffffffffu, timed_out) && (uint32_t)(b * B) < wlast) {
                     uint32_t hits = warp_block_hits(
                         S.rec[bf], 0, min(count, (int)(wlast - (uint32_t)(b * B))), lane, bx0, by0);
+                    // Gsem of this pixel and each Gaussian, loaded a Gaussian ahead:
+                    // issued before a pair's work and waited for after it (a load
+                    // waited for after alpha alone cost 4% of the kernel)
+                    float gsem = 0.f;
+                    if (hits)
+                        gsem = tmem_ld1_wait(tmem_ld1_issue(d1 + (uint32_t)(31 - __clz(hits))));
                     while (hits) {
                         const int j = 31 - __clz(hits);
                         hits ^= 1u << j;
                         const uint32_t pos = (uint32_t)(b * B + j);
                         const float* rc = &S.rec[bf][j][0];
-                        // Gsem of this pixel and Gaussian, loaded while alpha is evaluated
-                        const uint32_t gsem_raw = tmem_ld1_issue(d1 + (uint32_t)j);
+                        const uint32_t next_raw =
+                            tmem_ld1_issue(d1 + (uint32_t)(hits ? 31 - __clz(hits) : j));
                         float dx, dy, Gs, wq;
                         const float alpha = splat_alpha(rc, uf, vf, P.alpha_max, &dx, &dy, &Gs, &wq);
-                        const float gsem = tmem_ld1_wait(gsem_raw);
                         const bool contrib = !timed_out && pos < last && alpha >= P.alpha_min;
-                        if (!__any_sync(0xffffffffu, contrib)) continue;
-                        const float G_sem = gsem * ginv * finv;
-                        float gv[32];
-                        const float w = bwd_pair(rc, up, xt, yt, wq, dx, dy, alpha, Gs,
-                                                 contrib, G_sem, P.alpha_max, P.center_depth, T,
-                                                 Sacc, gv);
-                        if (contrib) {
-                            // w 2^14 = hi + lo, both float16, in W^T column j
-                            const float ws = w * W_SCALE;
-                            const __half wh = __float2half_rn(ws);
-                            const int off = wcol + (j >> 3) * Sm::SBO_W + (j & 7) * 16;
-                            *reinterpret_cast<__half*>(w0 + off) = wh;
-                            *reinterpret_cast<__half*>(w1 + off) =
-                                __float2half_rn(ws - __half2float(wh));
+                        if (__any_sync(0xffffffffu, contrib)) {
+                            const float G_sem = gsem * ginv * finv;
+                            float gv[32];
+                            const float w = bwd_pair(rc, up, xt, yt, wq, dx, dy, alpha, Gs,
+                                                     contrib, G_sem, P.alpha_max, P.center_depth, T,
+                                                     Sacc, gv);
+                            if (contrib) {
+                                // w 2^14 = hi + lo, both float16, in W^T column j
+                                const float ws = w * W_SCALE;
+                                const __half wh = __float2half_rn(ws);
+                                const int off = wcol + (j >> 3) * Sm::SBO_W + (j & 7) * 16;
+                                *reinterpret_cast<__half*>(w0 + off) = wh;
+                                *reinterpret_cast<__half*>(w1 + off) =
+                                    __float2half_rn(ws - __half2float(wh));
+                            }
+                            const uint32_t g = S.ids[gk & 3u][j];
+                            const size_t rix = (size_t)cam_idx * (size_t)P.n + g;
+                            // the warp's sum of component `lane`, added in float64
+                            // (see the FP32-pipe kernel)
+                            const float tot = warp_reduce_transpose32(gv, lane);
+                            if (tot != 0.f) atomicAdd(P.grec + rix * GREC_FLOATS + lane, (double)tot);
                         }
-                        const uint32_t g = S.ids[gk & 3u][j];
-                        const size_t rix = (size_t)cam_idx * (size_t)P.n + g;
-                        // the warp's sum of component `lane`, added in float64
-                        // (see the FP32-pipe kernel)
-                        const float tot = warp_reduce_transpose32(gv, lane);
-                        if (tot != 0.f) atomicAdd(P.grec + rix * GREC_FLOATS + lane, (double)tot);
+                        gsem = tmem_ld1_wait(next_raw);
                     }
                 }
                 // this warp is done with the batch's records, Gsem and W^T
