@@ -206,6 +206,9 @@ class Renderer:
                 abi.check(s, "unigs_bin_sort")
                 self.last_instances = need
                 return out
+            # the composite still reads the old workspace, which may belong to
+            # another stream than this one
+            torch.cuda.current_stream(self.device).synchronize()
             self._plan(int(need * 1.25) + 4096)
         raise RuntimeError("instance capacity could not be satisfied")
 
