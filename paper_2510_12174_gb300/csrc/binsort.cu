@@ -191,6 +191,7 @@ __global__ void __launch_bounds__(512)
                       unsigned long long* __restrict__ words, int64_t n_words,
                       unsigned long long* __restrict__ emit_words, int64_t n_emit_words,
                       uint2* __restrict__ ranges, int64_t n_tiles) {
+    pdl_begin();
     __shared__ uint32_t h[4][256];
     for (int j = threadIdx.x; j < 4 * 256; j += blockDim.x) (&h[0][0])[j] = 0;
     __syncthreads();
@@ -289,6 +290,7 @@ __device__ __forceinline__ uint32_t scan512(uint32_t v, uint32_t* wsum, uint32_t
 // tile.  KEYS: also write the keys (the last depth pass needs only the order).
 template <int PER, bool FROM_PAIRS, bool KEYS>
 __global__ void __launch_bounds__(RS_THREADS, 2) onesweep_kernel(const OnesweepParams P) {
+    pdl_begin();
     extern __shared__ __align__(16) unsigned char rs_raw[];
     OnesweepSmem<PER>& S = *reinterpret_cast<OnesweepSmem<PER>*>(rs_raw);
     constexpr int ITEMS = RS_THREADS * PER;
@@ -451,6 +453,7 @@ __device__ __forceinline__ int nth_bit(unsigned long long m, int r) {
 // 1.18 ms; with the list 0.034 + 0.051 ms).  Also counts the tile digits and clears the
 // look-back words of the chunks that its own instances start.
 __global__ void __launch_bounds__(256) emit_kernel(const EmitParams P) {
+    pdl_begin();
     __shared__ uint32_t hist[TILE_PASSES_MAX][RS_BINS];
     __shared__ uint32_t sw[32];
     __shared__ uint32_t s_chunk;
@@ -608,6 +611,7 @@ __global__ void __launch_bounds__(256) emit_kernel(const EmitParams P) {
 // largest rectangles stand together) go to different warps.
 constexpr int BIG_SEG = WIDE_TILES;
 __global__ void __launch_bounds__(256) emit_big_kernel(const EmitParams P, int max_segs) {
+    pdl_begin();
     __shared__ uint32_t hist[TILE_PASSES_MAX][RS_BINS];
     const int lane = threadIdx.x & 31;
     const int64_t n_big = P.st->n_big;
@@ -821,6 +825,7 @@ __global__ void __launch_bounds__(256)
 __global__ void __launch_bounds__(256)
     ranges_kernel(const uint32_t* __restrict__ keys, const WsHeader* __restrict__ hdr,
                   const SortState* __restrict__ st, uint2* __restrict__ ranges) {
+    pdl_begin();
     const uint32_t n = st->abort ? 0u : hdr->n_instances;
     // four tile ids per thread (the region is aligned to 256 bytes), and the
     // one before them
@@ -851,6 +856,7 @@ __global__ void __launch_bounds__(256)
 // the order inside a bucket is arbitrary and affects scheduling only).
 __global__ void __launch_bounds__(1024)
     tile_order_kernel(const uint2* __restrict__ ranges, int64_t n_tiles, uint32_t* __restrict__ order) {
+    pdl_begin();
     __shared__ uint32_t cnt[33];
     __shared__ uint32_t base[33];
     if (threadIdx.x < 33) cnt[threadIdx.x] = 0;
@@ -889,8 +895,8 @@ static void launch_onesweep(const OnesweepParams& P, int64_t n_max, cudaStream_t
     const int smem = (int)sizeof(OnesweepSmem<PER>);
     ensure_smem_limit(reinterpret_cast<const void*>(&onesweep_kernel<PER, FROM_PAIRS, KEYS>), smem);
     const int64_t chunks = (n_max + ITEMS - 1) / ITEMS, cap = (int64_t)sm_count() * 2;
-    onesweep_kernel<PER, FROM_PAIRS, KEYS>
-        <<<(unsigned)(chunks < cap ? chunks : cap), RS_THREADS, smem, st>>>(P);
+    launch_after(&onesweep_kernel<PER, FROM_PAIRS, KEYS>, chunks < cap ? chunks : cap, RS_THREADS,
+                 (size_t)smem, st, P);
 }
 
 template <bool FROM_PAIRS, bool KEYS>
@@ -990,7 +996,7 @@ int launch_bin_sort(const unigs_plan& p, void* ws, cudaStream_t st) {
         E.bits = tb;
         E.items = RS_THREADS * rs_per(p.capacity);
         const int64_t blocks = (total + 255) / 256, cap = (int64_t)sm_count() * 8;
-        emit_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, st>>>(E);
+        launch_after(&emit_kernel, blocks < cap ? blocks : cap, 256, 0, st, E);
         int max_tiles = 0;
         for (int k = 0; k < p.n_cams; ++k) {
             const int nt = p.tile_offset[k + 1] - p.tile_offset[k];
@@ -998,8 +1004,8 @@ int launch_bin_sort(const unigs_plan& p, void* ws, cudaStream_t st) {
         }
         launches += 1;
         if (max_tiles > MASK_TILES) {
-            emit_big_kernel<<<(unsigned)(blocks * 8 < cap ? blocks * 8 : cap), 256, 0, st>>>(
-                E, (max_tiles + BIG_SEG - 1) / BIG_SEG);
+            launch_after(&emit_big_kernel, blocks * 8 < cap ? blocks * 8 : cap, 256, 0, st, E,
+                         (max_tiles + BIG_SEG - 1) / BIG_SEG);
             ++launches;
         }
     }
@@ -1021,10 +1027,11 @@ int launch_bin_sort(const unigs_plan& p, void* ws, cudaStream_t st) {
     {
         const int64_t blocks = (p.capacity + 1023) / 1024;
         const int grid = (int)(blocks < 152 * 16 ? blocks : 152 * 16);
-        ranges_kernel<<<grid, 256, 0, st>>>(keys[0], hdr, ss, ranges);
+        launch_after(&ranges_kernel, grid, 256, 0, st, keys[0], hdr, ss, ranges);
         ++launches;
     }
-    tile_order_kernel<<<1, 1024, 0, st>>>(ranges, p.n_tiles, ws_ptr<uint32_t>(ws, p, OFF_ORDER));
+    launch_after(&tile_order_kernel, 1, 1024, 0, st, ranges, p.n_tiles,
+                 ws_ptr<uint32_t>(ws, p, OFF_ORDER));
     return launches + 1;
 }
 

@@ -252,6 +252,7 @@ __global__ void __launch_bounds__(256)
                       unsigned long long* __restrict__ masks, float* __restrict__ cull,
                       uint32_t* __restrict__ bits, int64_t n_bit_words,
                       WsHeader* __restrict__ hdr, uint32_t* __restrict__ kept_list) {
+    pdl_begin();
     const int64_t n = g.n;
     const int64_t total = n * (int64_t)n_cams;
     const int lane = threadIdx.x & 31;
@@ -407,6 +408,7 @@ __global__ void __launch_bounds__(256, 3)
                             float lowpass, const uint32_t* __restrict__ kept_list,
                             const WsHeader* __restrict__ hdr, float* __restrict__ rec,
                             float4* __restrict__ vp) {
+    pdl_begin();
     const int64_t n = g.n;
     const int64_t n_kept = hdr->n_kept;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n_kept;
@@ -552,6 +554,7 @@ __global__ void __launch_bounds__(256, 3)
 
 __global__ void init_kernel(CamTable tab, int n_cams, CamTable* __restrict__ dst,
                             WsHeader* __restrict__ hdr) {
+    pdl_begin();
     const int k = threadIdx.x;
     if (k < n_cams) dst->cam[k] = tab.cam[k];
     if (k == 0) {
@@ -636,17 +639,17 @@ int launch_preprocess(const unigs_plan& p, const unigs_gaussians& g, const CamTa
         const int64_t blocks = (total + 255) / 256;
         const int64_t cap = (int64_t)sm_count() * 64;
         const int grid = (int)(blocks < cap ? blocks : cap);
-        preprocess_kernel<<<grid, 256, 0, st>>>(
-            g, ws_ptr<CamTable>(ws, p, OFF_CAM), p.n_cams, p.cfg.tile_w, p.cfg.tile_h,
-            p.cfg.lowpass, ws_ptr<uint2>(ws, p, OFF_RECT), ws_ptr<uint32_t>(ws, p, OFF_TOUCH),
-            ws_ptr<uint32_t>(ws, p, OFF_ZBITS), cull_masks(ws, p), cull_records(ws, p),
-            cull_bits(ws, p), bit_word_count(p.capacity), hdr, kept_list);
+        launch_after(&preprocess_kernel, grid, 256, 0, st, g, ws_ptr<CamTable>(ws, p, OFF_CAM),
+                     p.n_cams, p.cfg.tile_w, p.cfg.tile_h, p.cfg.lowpass,
+                     ws_ptr<uint2>(ws, p, OFF_RECT), ws_ptr<uint32_t>(ws, p, OFF_TOUCH),
+                     ws_ptr<uint32_t>(ws, p, OFF_ZBITS), cull_masks(ws, p), cull_records(ws, p),
+                     cull_bits(ws, p), bit_word_count(p.capacity), hdr, kept_list);
         // grid-stride over the list, whose length only the device knows
         const int64_t cap2 = (int64_t)sm_count() * 32;
         const int grid2 = (int)(blocks < cap2 ? blocks : cap2);
-        preprocess_splat_kernel<<<grid2, 256, 0, st>>>(
-            g, ws_ptr<CamTable>(ws, p, OFF_CAM), p.cfg.lowpass, kept_list, hdr,
-            ws_ptr<float>(ws, p, OFF_REC), ws_ptr<float4>(ws, p, OFF_VP));
+        launch_after(&preprocess_splat_kernel, grid2, 256, 0, st, g,
+                     ws_ptr<CamTable>(ws, p, OFF_CAM), p.cfg.lowpass, kept_list, hdr,
+                     ws_ptr<float>(ws, p, OFF_REC), ws_ptr<float4>(ws, p, OFF_VP));
         launches += 2;
     }
     if (sem32_needed(p)) {
