@@ -92,12 +92,8 @@ __device__ __forceinline__ void accumulate_row(const float* row, float w, float 
     }
 }
 
-// CTAs per SM: the few logit accumulators of 8 channels leave 64 registers
-// enough, so four fit; more channels hold two.
-constexpr int fwd_ctas(int ns) { return ns <= 8 ? 4 : 2; }
-
 template <int NS, int B>
-__global__ void __launch_bounds__(256, fwd_ctas(NS)) render_fwd_kernel(const FwdParams P) {
+__global__ void __launch_bounds__(256, 2) render_fwd_kernel(const FwdParams P) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     FwdSmem<NS, B>& S = *reinterpret_cast<FwdSmem<NS, B>*>(smem_raw);
     const int tid = threadIdx.x;
@@ -317,9 +313,8 @@ int launch_render_fwd(const unigs_plan& p, const unigs_gaussians& g, void* ws,
     P.sem_bulk = (p.n_sem > 0) && ((p.n_sem * 4) % 16 == 0) &&
                  ((reinterpret_cast<uintptr_t>(P.sem) & 15) == 0);
     cudaMemsetAsync(P.work, 0, sizeof(uint32_t), st);
-    // forward shape fields, else batch 32 and as many CTAs as are resident
-    const int ctas = p.cfg.ctas_per_sm_fwd > 0 ? p.cfg.ctas_per_sm_fwd
-                                               : fwd_ctas(p.n_sem <= 8 ? 8 : 64);
+    // forward shape fields, else batch 32 x 2 CTAs per SM
+    const int ctas = p.cfg.ctas_per_sm_fwd > 0 ? p.cfg.ctas_per_sm_fwd : 2;
     const int batch = p.cfg.batch_fwd > 0 ? p.cfg.batch_fwd : 32;
     int64_t grid = (int64_t)sm_count() * ctas;
     if (grid > p.n_tiles) grid = p.n_tiles;
