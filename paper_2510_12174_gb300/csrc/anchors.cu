@@ -5,21 +5,22 @@
 // The five two-layer MLPs (F = H = 32) are about 11 k multiply-adds per anchor
 // forward and 32 k backward, in float32; at 100k anchors of 10 Gaussians with
 // 64 logits that is 30 and 90 us of the FP32 pipes, next to 35 and 70 us for
-// the bytes.  Each layer is a product of a weight matrix with a tile of TA
-// anchors: a block of 256 threads keeps the weights, the anchors' features and
-// one branch's hidden layer in shared memory (entries [unit][anchor]), and a
-// thread owns a register tile of 4 units x TA / 32 anchors, so that 8 16-byte
-// shared loads feed 64 multiply-adds.  Outputs go through shared memory, so
-// that a warp writes whole rows: with one thread per anchor (53 KB of weights
-// read by broadcast, one multiply-add per shared load) every store of a warp
-// fell into 32 different rows, and decode and backward took 913 and 1780 us
-// at that size.  Each output still sums its terms in the same order.
+// the bytes.  Each layer is a product of a weight matrix with a tile of 128 (or
+// 64, 32) anchors: a block keeps the weights, the anchors' features and one
+// branch's hidden layer in shared memory (entries [unit][anchor]), and a
+// thread owns a register tile of 4 units x 2 anchors.  Outputs and upstream
+// gradients go through shared memory, so that consecutive threads read and
+// write whole rows.  At that size decode takes 196 us and backward 530 us (913
+// and 1780 with one thread per anchor, whose stores fell into 32 rows a warp;
+// 236 and 941 with 8 warps of 4 x 4 tiles and global loads beside the
+// products).  What bounds them now: shared-memory operand reads (54% of peak)
+// and the latency between the phases of a tile.
 //
 // Backward: the same tiles give the outputs, dL/dh = W2^T g_y and dL/df = W1^T
 // g_pre; the parameter gradients dL/dW2 = sum_a g_y (x) h and dL/dW1 = sum_a
-// g_pre (x) f are 4 x 4 register tiles over the block's anchors, added to
-// accumulators in shared memory tile by tile; one float32 atomic per parameter
-// and block adds them at the end.
+// g_pre (x) f are register tiles over the block's anchors, added to
+// accumulators in shared memory tile by tile, then over a cluster of blocks in
+// float64; one float32 atomic per parameter and cluster adds them at the end.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
@@ -876,8 +877,8 @@ using Narrow = unigs::Tile<1, 256>;
 // Shared memory a block can have (sm_103a).
 constexpr size_t MAX_SMEM = 232448;
 
-// Anchors per tile / 32: 4 where that leaves every SM a tile and the buffers
-// fit, else 1, so that small sets still spread over the chip (a tile of 128
+// The wide tiles where that leaves every SM one of 128 anchors and the buffers
+// fit, else the narrow ones, so that small sets still spread over the chip (a tile of 128
 // takes about three times as long as one of 32).
 bool wide_tiles(int64_t n, size_t floats) {
     return n >= (int64_t)unigs::sm_count() * 128 && floats * sizeof(float) <= MAX_SMEM;
