@@ -111,7 +111,13 @@ class Renderer:
             self.cfg.flags |= abi.UNIGS_FLAG_CENTER_DEPTH
         self.device = scene.mean.device
         self.last_instances = None
-        self._hdr = None
+        # Where forward() reads the status block back.  Made here, so that no
+        # frame pays for it, and as a normal tensor whatever mode the renderer
+        # is built or first called in: it is written in place, which an
+        # inference tensor refuses outside inference mode.
+        with torch.inference_mode(False):
+            self._hdr = torch.empty(32, dtype=torch.uint8, pin_memory=True)
+        self._hdr_event = torch.cuda.Event()
         self._plan(capacity)
 
     # ------------------------------------------------------------------ plan
@@ -201,7 +207,9 @@ class Renderer:
             if not readback:
                 return out
             self._hdr_event.synchronize()
-            s, need = int(self._hdr_words[0]), int(self._hdr_need[0])
+            # status, instances (32 bits each), instances needed (64 bits)
+            hdr = self._hdr.numpy()
+            s, need = int(hdr.view(np.uint32)[0]), int(hdr.view(np.uint64)[1])
             if s != abi.UNIGS_ERR_CAPACITY:
                 abi.check(s, "unigs_bin_sort")
                 self.last_instances = need
@@ -214,11 +222,6 @@ class Renderer:
 
     def _copy_header(self):
         """Enqueues a copy of the workspace's status block to pinned memory."""
-        if self._hdr is None:
-            self._hdr = torch.empty(32, dtype=torch.uint8, pin_memory=True)
-            self._hdr_words = self._hdr.numpy().view(np.uint32)   # status, instances
-            self._hdr_need = self._hdr.numpy().view(np.uint64)[1:]
-            self._hdr_event = torch.cuda.Event()
         o = self.plan.off[0]
         self._hdr.copy_(self.ws[o: o + 32], non_blocking=True)
         self._hdr_event.record(torch.cuda.current_stream(self.device))

@@ -1,0 +1,34 @@
+"""Renderer.forward with its read-back of the status block."""
+import pytest
+import torch
+
+from paper_2510_12174_gb300 import rasterizer as rz
+from paper_2510_12174_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__ as ge
+    ge.build()
+    torch.cuda.set_device(0)
+
+
+def _room(seed):
+    return scenes.small_room(n=3000, width=64, height=52, n_sem=12, seed=seed)
+
+
+@pytest.mark.parametrize("build_inside", [False, True])
+def test_first_frame_in_inference_mode(build_inside):
+    """A renderer whose first frame is drawn in inference mode (an evaluation
+    before training) draws the next one outside it, and the other way round."""
+    sc, cams = _room(101)
+    with torch.inference_mode(build_inside):
+        r = rz.Renderer(rz.DeviceScene.from_scene(sc), cams)
+    with torch.inference_mode():
+        first = {k: v.clone() for k, v in r.forward().items()}
+    for mode in (False, True):
+        with torch.inference_mode(mode):
+            out = r.forward()
+            assert all(torch.equal(first[k], out[k]) for k in first)
