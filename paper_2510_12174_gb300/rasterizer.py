@@ -92,6 +92,37 @@ def _ptr(x: Optional[torch.Tensor]):
     return None if x is None else x.data_ptr()
 
 
+class _StatusBlock:
+    """Host copy of the status block at the start of a workspace.
+
+    Made with the renderer, so that no frame pays for it, and as a normal
+    tensor whatever mode the renderer is built or first called in: it is
+    written in place, which an inference tensor refuses outside inference
+    mode.  A deep copy of a renderer gets a block of its own (an event cannot
+    be copied).
+    """
+
+    BYTES = 32
+
+    def __init__(self):
+        with torch.inference_mode(False):
+            self.host = torch.empty(self.BYTES, dtype=torch.uint8, pin_memory=True)
+        self.event = torch.cuda.Event()
+
+    def __deepcopy__(self, memo):
+        return _StatusBlock()
+
+    def enqueue_copy(self, block: torch.Tensor):
+        self.host.copy_(block, non_blocking=True)
+        self.event.record(torch.cuda.current_stream(block.device))
+
+    def wait(self):
+        """(status, instances needed) once the copy has landed."""
+        self.event.synchronize()
+        h = self.host.numpy()
+        return int(h.view(np.uint32)[0]), int(h.view(np.uint64)[1])
+
+
 class Renderer:
     """Plans, owns the workspace and runs the forward / backward sequences.
 
@@ -111,13 +142,7 @@ class Renderer:
             self.cfg.flags |= abi.UNIGS_FLAG_CENTER_DEPTH
         self.device = scene.mean.device
         self.last_instances = None
-        # Where forward() reads the status block back.  Made here, so that no
-        # frame pays for it, and as a normal tensor whatever mode the renderer
-        # is built or first called in: it is written in place, which an
-        # inference tensor refuses outside inference mode.
-        with torch.inference_mode(False):
-            self._hdr = torch.empty(32, dtype=torch.uint8, pin_memory=True)
-        self._hdr_event = torch.cuda.Event()
+        self._status_block = _StatusBlock()
         self._plan(capacity)
 
     # ------------------------------------------------------------------ plan
@@ -195,7 +220,8 @@ class Renderer:
         for _ in range(4):
             self.preprocess_and_sort(readback=False)
             if readback:
-                self._copy_header()
+                o = self.plan.off[0]
+                self._status_block.enqueue_copy(self.ws[o: o + _StatusBlock.BYTES])
             st = self._stream()
             g = self.scene.struct()
             abi.check(abi.unigs_render_fwd(self.plan, g, self.ws.data_ptr(),
@@ -206,10 +232,7 @@ class Renderer:
                           "unigs_depth_normal_fwd")
             if not readback:
                 return out
-            self._hdr_event.synchronize()
-            # status, instances (32 bits each), instances needed (64 bits)
-            hdr = self._hdr.numpy()
-            s, need = int(hdr.view(np.uint32)[0]), int(hdr.view(np.uint64)[1])
+            s, need = self._status_block.wait()
             if s != abi.UNIGS_ERR_CAPACITY:
                 abi.check(s, "unigs_bin_sort")
                 self.last_instances = need
@@ -219,12 +242,6 @@ class Renderer:
             torch.cuda.current_stream(self.device).synchronize()
             self._plan(int(need * 1.25) + 4096)
         raise RuntimeError("instance capacity could not be satisfied")
-
-    def _copy_header(self):
-        """Enqueues a copy of the workspace's status block to pinned memory."""
-        o = self.plan.off[0]
-        self._hdr.copy_(self.ws[o: o + 32], non_blocking=True)
-        self._hdr_event.record(torch.cuda.current_stream(self.device))
 
     # -------------------------------------------------------------- backward
     def alloc_grads(self) -> Dict[str, torch.Tensor]:

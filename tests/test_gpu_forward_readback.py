@@ -1,4 +1,6 @@
 """Renderer.forward with its read-back of the status block."""
+import copy
+
 import pytest
 import torch
 
@@ -32,3 +34,17 @@ def test_first_frame_in_inference_mode(build_inside):
         with torch.inference_mode(mode):
             out = r.forward()
             assert all(torch.equal(first[k], out[k]) for k in first)
+
+
+def test_deep_copy_of_a_used_renderer():
+    """A deep copy draws the same frame, and re-plans on its own."""
+    sc, cams = _room(102)
+    r = rz.Renderer(rz.DeviceScene.from_scene(sc), cams)
+    out = r.forward()
+    q = copy.deepcopy(r)
+    capacity = r.capacity
+    q._plan(64)  # overflows: the copy reads its own status block and grows
+    for a in (q, r):
+        again = a.forward()
+        assert all(torch.equal(out[k], again[k]) for k in out)
+    assert r.capacity == capacity and q.capacity > 64
