@@ -212,26 +212,31 @@ class Renderer:
 
     def forward(self, out: Optional[Dict[str, torch.Tensor]] = None, readback: bool = True,
                 normal_d: bool = True) -> Dict[str, torch.Tensor]:
+        """Draws the cameras into ``out`` (allocated when None).
+
+        With ``readback`` a frame that exceeds the capacity is drawn again with
+        a larger plan, and an error status raises.  What ``out`` then holds is
+        undefined, but for a non-finite parameter (UNIGS_FLAG_CHECK_FINITE): it
+        raises before the caller's ``out`` is written.  A renderer draws one
+        frame at a time: its workspace and status block are not shared between
+        threads or streams.
+        """
+        wait_first = readback and out is not None and \
+            self.cfg.flags & abi.UNIGS_FLAG_CHECK_FINITE
         out = out if out is not None else self.alloc_outputs()
-        # With a read-back, the composite is enqueued before the instance count
-        # is waited for (over the capacity it renders nothing, and the sequence
-        # runs again with a larger plan): waiting first left the GPU idle for
-        # 45 us between the sort and the composite of every frame.
+        if not readback or wait_first:
+            self.preprocess_and_sort(readback)
+            self._composite(out, normal_d)
+            return out
+        # The composite is enqueued before the instance count is waited for
+        # (over the capacity it renders nothing, and the sequence runs again
+        # with a larger plan): waiting first left the GPU idle for 45 us between
+        # the sort and the composite of every frame.
         for _ in range(4):
             self.preprocess_and_sort(readback=False)
-            if readback:
-                o = self.plan.off[0]
-                self._status_block.enqueue_copy(self.ws[o: o + _StatusBlock.BYTES])
-            st = self._stream()
-            g = self.scene.struct()
-            abi.check(abi.unigs_render_fwd(self.plan, g, self.ws.data_ptr(),
-                                           self._out_struct(out), st), "unigs_render_fwd")
-            if normal_d:
-                abi.check(abi.unigs_depth_normal_fwd(self.plan, self.cams, _ptr(out["depth"]),
-                                                     _ptr(out["normal_d"]), st),
-                          "unigs_depth_normal_fwd")
-            if not readback:
-                return out
+            o = self.plan.off[0]
+            self._status_block.enqueue_copy(self.ws[o: o + _StatusBlock.BYTES])
+            self._composite(out, normal_d)
             s, need = self._status_block.wait()
             if s != abi.UNIGS_ERR_CAPACITY:
                 abi.check(s, "unigs_bin_sort")
@@ -242,6 +247,16 @@ class Renderer:
             torch.cuda.current_stream(self.device).synchronize()
             self._plan(int(need * 1.25) + 4096)
         raise RuntimeError("instance capacity could not be satisfied")
+
+    def _composite(self, out: Dict[str, torch.Tensor], normal_d: bool):
+        st = self._stream()
+        g = self.scene.struct()
+        abi.check(abi.unigs_render_fwd(self.plan, g, self.ws.data_ptr(), self._out_struct(out), st),
+                  "unigs_render_fwd")
+        if normal_d:
+            abi.check(abi.unigs_depth_normal_fwd(self.plan, self.cams, _ptr(out["depth"]),
+                                                 _ptr(out["normal_d"]), st),
+                      "unigs_depth_normal_fwd")
 
     # -------------------------------------------------------------- backward
     def alloc_grads(self) -> Dict[str, torch.Tensor]:

@@ -4,6 +4,7 @@ import copy
 import pytest
 import torch
 
+from paper_2510_12174_gb300 import abi
 from paper_2510_12174_gb300 import rasterizer as rz
 from paper_2510_12174_gb300 import scenes
 
@@ -48,3 +49,23 @@ def test_deep_copy_of_a_used_renderer():
         again = a.forward()
         assert all(torch.equal(out[k], again[k]) for k in out)
     assert r.capacity == capacity and q.capacity > 64
+
+
+def test_non_finite_parameter_leaves_the_callers_frame():
+    """With the check on, a non-finite opacity raises before the caller's
+    buffers are written."""
+    sc, cams = _room(103)
+    cfg = abi.unigs_config_default()
+    cfg.flags |= abi.UNIGS_FLAG_CHECK_FINITE
+    scene = rz.DeviceScene.from_scene(sc)
+    r = rz.Renderer(scene, cams, cfg=cfg)
+    out = r.forward()
+    before = {k: v.clone() for k, v in out.items()}
+    good = scene.opacity.clone()
+    scene.opacity[::2] = float("nan")
+    with pytest.raises(RuntimeError):
+        r.forward(out)
+    torch.cuda.synchronize()
+    assert all(torch.equal(before[k], out[k]) for k in out)
+    scene.opacity.copy_(good)
+    assert all(torch.equal(before[k], v) for k, v in r.forward(out).items())
