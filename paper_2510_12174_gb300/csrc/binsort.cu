@@ -30,6 +30,7 @@
 // 1280x720 view of 1M, 2.7M instances, 0.36 -> 0.22 ms; one 256x256 view of
 // 10k, 0.33 -> 0.24 ms for the whole frame.
 #include "launch.h"
+#include "lookback.cuh"
 
 namespace unigs {
 
@@ -128,8 +129,7 @@ int scan_u32(const uint32_t* in, int64_t n, uint32_t* partial, uint32_t* out, ui
 }
 
 // ------------------------------------------------------- single-kernel passes
-// A look-back word: (epoch << 2 | state) << 32 | count.  state 1: the chunk's
-// own count, 2: its inclusive prefix; any other epoch: not written yet.
+// Stores a look-back word (look_back_walk has its layout).
 __device__ __forceinline__ void lb_store(unsigned long long* w, uint32_t epoch, uint32_t state,
                                          uint32_t count) {
     const unsigned long long v = ((unsigned long long)(epoch << 2 | state) << 32) | count;
@@ -146,40 +146,15 @@ __device__ __forceinline__ void emit_store(unsigned long long* w, unsigned long 
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"(v) : "memory");
 }
 
-constexpr uint32_t LB_WAIT_LIMIT = 1u << 20;  // polls of one word, about a second
+constexpr uint32_t LB_WAIT_LIMIT = 1u << 20;  // polls of one unwritten word, about a second
 constexpr int LB_WIDE = 8;                    // predecessors read per step
 
-// Sum of the counts of chunks [0, chunk) in column `col` of the look-back
-// table (rows of `stride` words).  Reads LB_WIDE predecessors at a time: one
-// memory latency per step, where one at a time a full first wave of chunks
-// would pay a latency per chunk.  Returns false when a wait gave up.
+// look_back_walk over column `col` of the look-back table (rows of `stride` words).
 __device__ __forceinline__ bool look_back(const unsigned long long* words, int64_t chunk,
                                           int stride, int col, uint32_t epoch, uint32_t* sum_out) {
-    uint32_t sum = 0, polls = 0;
-    int64_t p = chunk - 1;
-    while (p >= 0) {
-        unsigned long long v[LB_WIDE];
-#pragma unroll
-        for (int j = 0; j < LB_WIDE; ++j)
-            v[j] = p - j >= 0 ? lb_load(words + (p - j) * stride + col) : 0ull;
-        int used = 0;
-        bool open = true, found = false;
-#pragma unroll
-        for (int j = 0; j < LB_WIDE; ++j) {
-            const uint32_t tag = (uint32_t)(v[j] >> 32);
-            open = open && !found && p - j >= 0 && (tag >> 2) == epoch && (tag & 3u) != 0u;
-            if (open) {
-                sum += (uint32_t)v[j];
-                found = (tag & 3u) == 2u;
-                ++used;
-            }
-        }
-        if (found) break;
-        p -= used;
-        if (used == 0 && ++polls > LB_WAIT_LIMIT) return false;
-    }
-    *sum_out = sum;
-    return true;
+    return look_back_walk<LB_WIDE>(
+        [&](int64_t p) { return lb_load(words + p * stride + col); }, chunk, epoch, LB_WAIT_LIMIT,
+        sum_out);
 }
 
 // Digit counts of the depth keys of the pairs with a kept tile, for all four
@@ -487,7 +462,7 @@ __global__ void __launch_bounds__(256) emit_kernel(const EmitParams P) {
             unsigned long long* w = P.emit_words;
             bool bad = false;
             if (lane == 0) emit_store(w + chunk, (chunk == 0 ? 2ull : 1ull) << 62 | tot);
-            uint32_t polls = 0;
+            PollLimit wait(LB_WAIT_LIMIT);
             for (int64_t p = chunk - 1; p >= 0;) {
                 // lane l: predecessors p - 2 l and p - 2 l - 1
                 const int64_t p0 = p - 2 * lane;
@@ -506,12 +481,14 @@ __global__ void __launch_bounds__(256) emit_kernel(const EmitParams P) {
                 base += c;
                 if (at == 32) {
                     p -= 64;
+                    wait.give_up(true);
                     continue;
                 }
                 const int a0 = __shfl_sync(0xffffffffu, s0, at), a1 = __shfl_sync(0xffffffffu, s1, at);
                 if (a0 == 2 || (a0 == 1 && a1 == 2)) break;
-                p -= 2 * at + (a0 == 1 ? 1 : 0);  // the unwritten word is read again
-                if (++polls > LB_WAIT_LIMIT) {
+                const int used = 2 * at + (a0 == 1 ? 1 : 0);
+                p -= used;  // the unwritten word is read again
+                if (wait.give_up(used > 0)) {
                     bad = true;
                     break;
                 }
