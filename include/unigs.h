@@ -197,7 +197,8 @@ typedef struct {
     int64_t n_pixels;       /* all cameras */
     int32_t tile_offset[UNIGS_MAX_CAMS + 1];
     int64_t pixel_offset[UNIGS_MAX_CAMS + 1];
-    int32_t sort_passes;    /* 8-bit digits of the used (tile, depth) key bits */
+    int32_t sort_passes;    /* radix passes of the binning: 4 by depth, then by
+                               tile, up to 9 bits each */
     int32_t reserved;
     size_t ws_bytes;
     size_t off[20];         /* internal region offsets */

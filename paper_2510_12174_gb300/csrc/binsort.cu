@@ -920,7 +920,7 @@ int launch_bin_sort(const unigs_plan& p, void* ws, cudaStream_t st) {
     P.words = words;
     P.st = ss;
     P.hdr = hdr;
-    for (int pass = 0; pass < 4; ++pass) {
+    for (int pass = 0; pass < DEPTH_PASSES; ++pass) {
         const int src = (pass & 1) ^ 1, dst = src ^ 1;
         P.kin = pass ? dz[src] : zbits;
         P.vin = pass ? dt[src] : touched;
@@ -935,16 +935,14 @@ int launch_bin_sort(const unigs_plan& p, void* ws, cudaStream_t st) {
         P.epoch = 1u + pass;
         if (pass == 0)
             launch_onesweep_n<true, true>(P, total, st);
-        else if (pass < 3)
+        else if (pass < DEPTH_PASSES - 1)
             launch_onesweep_n<false, true>(P, total, st);
         else
             launch_onesweep_n<false, false>(P, total, st);
         ++launches;
     }
-    int tile_bits = 0;
-    while (((int64_t)1 << tile_bits) < p.n_tiles) ++tile_bits;
-    const int tpasses = (tile_bits + 8) / 9;
-    const int tb = tpasses ? (tile_bits + tpasses - 1) / tpasses : 0;
+    const int tpasses = tile_pass_count(p.n_tiles);
+    const int tb = tpasses ? (tile_id_bits(p.n_tiles) + tpasses - 1) / tpasses : 0;
     uint32_t* keys[2] = {ws_ptr<uint32_t>(ws, p, OFF_KEYS0), ws_ptr<uint32_t>(ws, p, OFF_KEYS1)};
     uint32_t* vals[2] = {ws_ptr<uint32_t>(ws, p, OFF_VALS0), ws_ptr<uint32_t>(ws, p, OFF_VALS1)};
     // the last tile pass writes buffer 0

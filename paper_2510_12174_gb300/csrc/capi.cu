@@ -202,9 +202,7 @@ unigs_status unigs_plan_init(unigs_plan* plan, const unigs_gaussians* g, const u
     int64_t cap = instance_capacity ? instance_capacity : 4 * total;
     if (cap > 0x7fffffffLL) cap = 0x7fffffffLL;
     plan->capacity = cap;
-    int tile_bits = 0;
-    while (((int64_t)1 << tile_bits) < tiles) ++tile_bits;
-    plan->sort_passes = (32 + tile_bits + 7) / 8;
+    plan->sort_passes = DEPTH_PASSES + tile_pass_count(tiles);
 
     // look-back words of the radix passes: 256 a chunk of pairs, 512 a chunk of
     // instances
@@ -358,13 +356,10 @@ unigs_status unigs_stats_poll(const unigs_plan* plan, const void* ws, int64_t* p
 
 int32_t unigs_launches_per_step(const unigs_plan* plan) {
     if (!plan) return 0;
-    int tile_bits = 0;
-    while (((int64_t)1 << tile_bits) < plan->n_tiles) ++tile_bits;
     int emits = 1;
     for (int k = 0; k < plan->n_cams; ++k)
         if (plan->tile_offset[k + 1] - plan->tile_offset[k] > MASK_TILES) emits = 2;
-    const int bin = 1 /*depth digits*/ + 4 /*depth passes*/ + emits +
-                    (tile_bits + 8) / 9 /*tile passes*/ + 1 /*ranges*/ + 1 /*tile order*/;
+    const int bin = 1 /*depth digits*/ + plan->sort_passes + emits + 1 /*ranges*/ + 1 /*tile order*/;
     int conv = 0;
     if (sem32_needed(*plan)) {
         const int64_t cnt = plan->n * (int64_t)plan->n_sem;

@@ -261,7 +261,15 @@ constexpr int RS_PER_LARGE = 16, RS_PER_SMALL = 4;
 __host__ __device__ constexpr int rs_per(int64_t n) {
     return n >= 4 * 1000 * 1000 ? RS_PER_LARGE : RS_PER_SMALL;
 }
+constexpr int DEPTH_PASSES = 4;     // 32 depth bits, 8 at a time
 constexpr int TILE_PASSES_MAX = 4;  // ceil(31 tile bits / 9)
+// Bits of a tile id, and the passes that sort by them (digits of at most 9 bits).
+__host__ inline int tile_id_bits(int64_t n_tiles) {
+    int bits = 0;
+    while (((int64_t)1 << bits) < n_tiles) ++bits;
+    return bits;
+}
+__host__ inline int tile_pass_count(int64_t n_tiles) { return (tile_id_bits(n_tiles) + 8) / 9; }
 constexpr int TICKET_EMIT = 4;      // tickets 0..3: depth passes, then emission, tile passes
 
 // State of one binning, zeroed at its start.
