@@ -82,7 +82,9 @@ typedef struct {
 } unigs_camera;
 
 /* The Gaussian map G = {mu, q, s, alpha, h, o, k} of Eq. 1, device pointers.
- * mean [3][n], quat [4][n] (w,x,y,z; need not be unit), scale [3][n] (> 0),
+ * mean [3][n], quat [4][n] (w,x,y,z; need not be unit), scale [3][n] (> 0;
+ * the composites square its reciprocal in float32 without subnormals, which
+ * holds from 2^-50 to 2^50 of the scene's unit),
  * opacity [n] (already activated, in (0,1)), kfac [n], sh [n][(deg+1)^2][3],
  * sem [n][n_sem].  sh and sem are float32 (feat_dtype 0) or bfloat16
  * (feat_dtype 1); every other array is float32.  All pointers 16-byte
@@ -146,7 +148,9 @@ typedef struct {
  * paper does not print its values), and 0 (= the library's choice) for every
  * launch-shape field.  unigs_plan_init rejects settings outside
  * 0 <= alpha_min <= alpha_max < 1 (the backward divides by 1 - alpha),
- * 0 <= T_min < 1 and a finite lowpass >= 0.  The launch shape changes the speed only: the forward
+ * 0 <= T_min < 1 and a finite lowpass >= 0.  The backward restores a
+ * transmittance with the rounding of a float32 division; where T_min lets it
+ * fall below 2^-102, to 2 units of the last place.  The launch shape changes the speed only: the forward
  * outputs do not depend on it (the tensor-core logit blend: up to float32
  * summation order), the gradients up to float32 atomic summation order. */
 typedef struct {

@@ -31,6 +31,20 @@ __device__ __forceinline__ void cross_acc(const float* a, const float* b, float*
     c[2] += a[0] * b[1] - a[1] * b[0];
 }
 
+// T / om, rom the approximate reciprocal of om in [2^-24, 1] (om = 1 - alpha,
+// alpha <= alpha_max < 1).  A Newton step rounds the reciprocal correctly but
+// for cases within 2^-20 of a tie; with the quotient's residual, exact by the
+// fused multiply-add, the corrected quotient is then the rounded one
+// (Markstein 1990), in four instructions and without the range tests of a
+// general division.  T is in [T_min, 1]; only a T_min below 2^-102 lets T fall
+// where the residual underflows.  The quotient is then up to 2 units of the
+// last place off, of a T that the forward already rounded in that range.
+__device__ __forceinline__ float restored_T(float T, float om, float rom) {
+    const float y = __fmaf_rn(__fmaf_rn(-om, rom, 1.f), rom, rom);
+    const float q = __fmul_rn(T, y);
+    return __fmaf_rn(__fmaf_rn(-om, q, T), y, q);
+}
+
 // One pair of the reverse walk.  With w_i = alpha_i T_i,
 // G_i = upstream gradient . features of Gaussian i (G_sem its logit part) and
 // S_i = sum_{j>i} w_j G_j (Sacc),
@@ -46,21 +60,12 @@ __device__ __forceinline__ float bwd_pair(const float* __restrict__ rc, const Pi
                                           float G_sem, float alpha_max, int center_depth,
                                           float& T, float& Sacc, float (&gv)[32]) {
     const float om = 1.f - alpha;
-    // om >= 1 - alpha_max.  The restoration T <- T / om runs along
-    // the whole list, so it takes the correctly rounded quotient
-    // (with an approximate one the worst cancelling rotation
-    // gradient of a 200k-Gaussian test scene drifted 2.5x further
-    // from the float64 reference); dL/dalpha takes the approximate
-    // reciprocal.  A Newton step rounds the reciprocal correctly but
-    // for cases within 2^-20 of a tie; with the quotient's residual,
-    // exact by the fused multiply-add, the corrected quotient is then
-    // the rounded one (Markstein 1990).  T is in [T_min, 1] and om in
-    // [1 - alpha_max, 1], so the range tests of a general division
-    // have nothing to find.
+    // The restoration T <- T / om runs along the whole list, so it takes the
+    // correctly rounded quotient (with an approximate one the worst cancelling
+    // rotation gradient of a 200k-Gaussian test scene drifted 2.5x further
+    // from the float64 reference); dL/dalpha takes the approximate reciprocal.
     const float rom = rcp_ftz(om);
-    const float ryn = __fmaf_rn(__fmaf_rn(-om, rom, 1.f), rom, rom);
-    const float q0 = __fmul_rn(T, ryn);
-    const float Tq = __fmaf_rn(__fmaf_rn(-om, q0, T), ryn, q0);
+    const float Tq = restored_T(T, om, rom);
     if (contrib) T = Tq;
     const float w = contrib ? alpha * T : 0.f;
     PairGeom G;
