@@ -69,3 +69,18 @@ def test_non_finite_parameter_leaves_the_callers_frame():
     assert all(torch.equal(before[k], out[k]) for k in out)
     scene.opacity.copy_(good)
     assert all(torch.equal(before[k], v) for k, v in r.forward(out).items())
+
+
+def test_overflow_on_a_side_stream():
+    """A frame over the capacity is drawn again on the stream it was asked for
+    on, whatever stream the first workspace came from."""
+    sc, cams = _room(104)
+    ref = rz.Renderer(rz.DeviceScene.from_scene(sc), cams).forward()
+    r = rz.Renderer(rz.DeviceScene.from_scene(sc), cams, capacity=64)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        out = r.forward()
+        assert r.capacity > 64
+    side.synchronize()
+    assert all(torch.equal(ref[k], out[k]) for k in ref)
