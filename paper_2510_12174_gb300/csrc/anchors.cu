@@ -13,8 +13,8 @@
 // write whole rows.  At that size decode takes 196 us and backward 530 us (913
 // and 1780 with one thread per anchor, whose stores fell into 32 rows a warp;
 // 236 and 941 with 8 warps of 4 x 4 tiles and global loads beside the
-// products).  What bounds them now: shared-memory operand reads (54% of peak)
-// and the latency between the phases of a tile.
+// products).  What bounds them now: shared-memory operand reads (55% of peak in
+// decode, 45% in backward) and the latency between the phases of a tile.
 //
 // Backward: the same tiles give the outputs, dL/dh = W2^T g_y and dL/df = W1^T
 // g_pre; the parameter gradients dL/dW2 = sum_a g_y (x) h and dL/dW1 = sum_a
@@ -67,8 +67,9 @@ struct DecodeOut {
     void *sh, *sem;
 };
 
-// i / d for 0 <= i < 2^16, 1 <= d <= 192, inv = 1.f / d: the product is within
-// 2^-22 of (i + 1/2) / d, which is at least 1 / (2 d) from an integer.  Three
+// i / d for 0 <= i < 2^16, 1 <= d <= 192, inv = 1.f / d: the product of the two
+// rounded factors is (i + 1/2) / d to a relative 2^-22, so at most 2^-6 / d off,
+// where the exact value is at least 1 / (2 d) from an integer.  Three
 // instructions against some twenty for a division by a runtime integer, one or
 // two of which stood beside every output.
 struct FastDiv {

@@ -12,13 +12,14 @@
 // normal flow to the per-(camera, Gaussian) ray-ellipsoid setup (M_c, v_s,
 // N_w); dL/dalpha flows to opacity, conic and projected centre.  The 32
 // lanes of a warp (32 pixels) are summed with a butterfly transpose-reduction
-// (lane L ends with component L) before one float32 atomic per lane.  The
+// (lane L ends with component L) before one float64 atomic per lane.  The
 // semantic gradients sum_l w_l g_O,l of the warp's 32 pixels are gathered
 // densely from the tile's upstream-gradient rows in shared memory (4 channels
 // per 16-byte load, w = 0 for pixels that do not contribute), one 16-byte
 // atomic per 4 channels.
 //
-// Kernel 2, one thread per Gaussian, loops over the cameras: conic -> 2D
+// Kernel 2, a warp per 32 Gaussians whose (camera, Gaussian) pairs are dealt to
+// its lanes, maps each record onto the parameters: conic -> 2D
 // covariance -> (J, Sigma) -> mean, rotation, scale (EWA chain of 3DGS);
 // M_c = S^-1 R^T R_cw, v_s = S^-1 R^T (C - mu), N_w = R S^-1 -> R, s, mu
 // (supplement Sec. 2: dL/ds_k = -(g_vs,k v_s,k + g_ds,k d_s,k)/s_k per ray,

@@ -110,17 +110,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// One float32 column of this thread's tensor-memory lane.
-__device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
-    uint32_t r;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    return __uint_as_float(r);
-}
-
-// A tensor-memory load issued early and waited for later: the wait takes the
-// destination register as an operand, so it stays allocated (and is not read)
-// until the load has landed.
+// One float32 column of this thread's tensor-memory lane, issued early and
+// waited for later: the wait takes the destination register as an operand, so it
+// stays allocated (and is not read) until the load has landed.  That holds
+// while the compiler keeps it in a register: a kernel that spilled it in between
+// would store a value that has not landed.  The tensor-core backward, which holds
+// one across a pair's work, compiles without spills for every width, and has to.
 __device__ __forceinline__ uint32_t tmem_ld1_issue(uint32_t taddr) {
     uint32_t r;
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
