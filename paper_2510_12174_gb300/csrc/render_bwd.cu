@@ -547,22 +547,16 @@ __global__ void __launch_bounds__(PREBWD_THREADS, 4) preprocess_bwd_kernel(const
                     sh_eval_basis_grad(d[0], d[1], d[2], DEG, dY);
                     float g_dir[3] = {0.f, 0.f, 0.f};
                     const size_t shb = (size_t)i * n_sh * 3;
-                    // rows of 4 or 16 coefficients are whole words: 3 or 12 vector
-                    // loads, where an element per load cost a sector each
-                    float hv[3 * n_sh];
-                    if constexpr (3 * n_sh % 4 == 0)
-                        load_feats<3 * n_sh>(P.g.sh, shb, P.g.feat_dtype, hv);
-                    else
-#pragma unroll
-                        for (int e = 0; e < 3 * n_sh; ++e)
-                            hv[e] = load_feat(P.g.sh, shb + e, P.g.feat_dtype);
+                    // an element per load: vector loads take 0.1% off a training
+                    // iteration, but with them the compiled kernel adds the shares
+                    // of a Gaussian seen by three cameras or more in another order
 #pragma unroll
                     for (int ch = 0; ch < 3; ++ch) {
                         float hc[n_sh];
                         float raw = 0.5f;
 #pragma unroll
                         for (int kk = 0; kk < n_sh; ++kk) {
-                            hc[kk] = hv[3 * kk + ch];
+                            hc[kk] = load_feat(P.g.sh, shb + kk * 3 + ch, P.g.feat_dtype);
                             raw = fmaf(Y[kk], hc[kk], raw);
                         }
                         if (raw < 0.f) continue;  // clamped at 0
